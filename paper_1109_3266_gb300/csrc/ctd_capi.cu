@@ -222,7 +222,6 @@ void fill_request(Phantom &P, uint64_t seed, ctd::RequestDesc &q)
 {
     std::memset(&q, 0, sizeof(q));
     q.vox = P.vox.p;
-    q.unused = nullptr;
     q.tab = P.tab.p;
     q.mmax = P.mm.p;
     q.rsurf = P.rs.p;
@@ -252,6 +251,8 @@ void fill_request(Phantom &P, uint64_t seed, ctd::RequestDesc &q)
     q.nx = P.nx;
     q.ny = P.ny;
     q.nz = P.nz;
+    q.nxy = static_cast<uint32_t>(P.nx) * static_cast<uint32_t>(P.ny);
+    q.idx0 = 0u - ctd::kTruncPattern * (1u + static_cast<uint32_t>(P.nx) + q.nxy);
     q.fnx = static_cast<float>(P.nx);
     q.fny = static_cast<float>(P.ny);
     q.fnz = static_cast<float>(P.nz);
@@ -294,6 +295,8 @@ void fill_shared(Phantom &P, ctd::SharedTables &sh)
     sh.n_zeta = P.phys.n_zeta;
     sh.e_min = P.phys.e_min_kev;
     sh.max_n_mat = static_cast<int>(P.mats.size());
+    sh.cells = static_cast<uint32_t>(P.n_e - 1) * static_cast<uint32_t>(P.phys.n_zeta - 1);
+    sh.wide = ctd::wide_index(P.nx, P.ny, P.nz, sh.max_n_mat, P.n_e, P.phys.n_zeta);
 }
 
 cudaEvent_t event_at(ctd_ctx *ctx, size_t i)

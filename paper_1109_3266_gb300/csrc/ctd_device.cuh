@@ -73,10 +73,22 @@ __device__ __forceinline__ U4 block(uint64_t seed, uint64_t h, uint32_t step, ui
 // a = 1 + k 2^-23 (k = x >> 9 as the significand) minus (1 - 2^-24) is
 // (2k + 1) 2^-24 exactly (2k + 1 < 2^24 fits the significand, so the one
 // subtraction does not round): the same value without an integer conversion.
+// One funnel shift of (127 : x) by 9 puts the exponent 127 above x >> 9.
 __device__ __forceinline__ float uni(uint32_t x)
 {
-    return __uint_as_float((x >> 9) | 0x3f800000u) - 0x1.fffffep-1f;
+    return __uint_as_float(__funnelshift_r(x, 127u, 9)) - 0x1.fffffep-1f;
 }
+
+// trunc(f) + 2^23 for 0 <= f < 2^23, in one full-rate addition rounded toward
+// zero (a conversion instruction runs at a quarter of the rate): its bit pattern
+// is kTruncBits + trunc(f), and taking 2^23 off again is exact.
+constexpr float kTrunc = 8388608.0f;
+constexpr uint32_t kTruncBits = kTruncPattern;
+__device__ __forceinline__ float trunc_up(float f) { return __fadd_rz(f, kTrunc); }
+
+// 2^kRhoExpBias, which takes a packed density back to its value
+constexpr float kRhoScale = 0x1p108f;
+static_assert(kRhoExpBias == 108, "kRhoScale is 2^kRhoExpBias");
 
 // ---------------------------------------------------------------- log and sincos
 // The hardware approximations (the SFU's base-2 logarithm and sine/cosine).
@@ -124,10 +136,6 @@ __device__ __forceinline__ float trunc32(double d)
 // e = -d/2 of one Newton step c = 1.5 - 0.5 n2 for 1/sqrt(n2) from 1 is d
 // truncated to binary32 times -1/2, applied to each component with one fused
 // multiply-add.
-// Bound by issue slots and by the wait for the narrow FP64 pipe, not by its rate:
-// the widening and truncation around the three multiply-adds were some forty
-// instructions with branches, now fifteen without.  CBCT water, 2e8 histories:
-// transport 18.44 -> 16.88 ms; head 30.12 -> 28.67 ms; results bit-identical.
 __device__ __forceinline__ void renorm(float &ux, float &uy, float &uz)
 {
     const double dx = widen_abs(ux), dy = widen_abs(uy), dz = widen_abs(uz);
@@ -197,27 +205,26 @@ __device__ __forceinline__ void rotate(float &ux, float &uy, float &uz, float mu
     renorm(ux, uy, uz);
 }
 
-// energy node j and fraction te on the 1 keV grid
+// energy node j and fraction te on the 1 keV grid (e >= e_min, n_e <= 10^5)
 __device__ __forceinline__ int enode(float e, int e_min, int n_e, float &te)
 {
     const float fe = e - static_cast<float>(e_min);
-    int j = static_cast<int>(fe);
-    if (j > n_e - 2) j = n_e - 2;
-    if (j < 0) j = 0;
-    te = fe - static_cast<float>(j);
-    return j;
+    const float t = fminf(trunc_up(fe), kTrunc + static_cast<float>(n_e - 2));
+    te = fe - (t - kTrunc);
+    return static_cast<int>(__float_as_uint(t) - kTruncBits);
 }
 
-// bilinear lookup of mu(zeta, E) on a surface (Sec. 2.2.2); S holds the surface as
-// cells of the four corners of a lookup, [n_e - 1][n_zeta - 1] float4, so one
-// 16-byte read fetches them
-__device__ __forceinline__ float surface(const float *__restrict__ S, int n_zeta, int j, float te, float z)
+// bilinear lookup of mu(zeta, E) (Sec. 2.2.2) on a surface whose row j of cells
+// starts at S; a surface is held as cells of the four corners of a lookup,
+// [n_e - 1][n_zeta - 1] float4, so one 16-byte read fetches them.  Cell is
+// uint32_t where every cell index of the launch fits, else size_t.
+template <class Cell>
+__device__ __forceinline__ float surface(const float *__restrict__ S, Cell row, int n_zeta, float te, float z)
 {
     const float zf = __fmul_rn(z, static_cast<float>(n_zeta - 1));   // rounded on its own, never fused
-    int i = static_cast<int>(zf);
-    if (i > n_zeta - 2) i = n_zeta - 2;
-    const float a = zf - static_cast<float>(i);
-    const float4 c = __ldg(reinterpret_cast<const float4 *>(S) + (static_cast<size_t>(j) * (n_zeta - 1) + i));
+    const float t = fminf(trunc_up(zf), kTrunc + static_cast<float>(n_zeta - 2));
+    const float a = zf - (t - kTrunc);
+    const float4 c = __ldg(reinterpret_cast<const float4 *>(S) + (row + (__float_as_uint(t) - kTruncBits)));
     const float a0 = c.x, a1 = c.y, b0 = c.z, b1 = c.w;
     const float lo = __fmaf_rn(a, a1 - a0, a0);
     const float hi = __fmaf_rn(a, b1 - b0, b0);

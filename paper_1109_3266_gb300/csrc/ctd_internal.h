@@ -89,7 +89,7 @@ enum { kCntPe = 0, kCntCompton, kCntRayleigh, kCntFict, kCntEscaped, kCntMissed,
 // request it is working on into shared memory.
 struct alignas(16) RequestDesc {
     const uint32_t *vox;         // [nvox] material and density of each voxel, one word (kRhoExpBias)
-    const void *unused;          // keeps the descriptor a whole number of 16-byte words
+    uint32_t nxy, idx0;          // nx * ny and -kTruncBits (1 + nx + nxy) mod 2^32 (the voxel index from truncated positions)
     const float *tab;            // [n_mat][n_e][4]: c1, c2, c3 (cm^2/g), c3[j+1] - c3[j] in binary32
     const float *mmax;           // [n_e] majorant mu_max(E), 1/cm
     // R and C surfaces as cells of 4 floats, [n_e - 1][n_zeta - 1] per surface: cell (j, i)
@@ -140,6 +140,10 @@ constexpr int kMaxPhantomMaterials = 16;
 constexpr uint32_t kRhoExpBias = 108;
 constexpr uint32_t kRhoExpLo = 109, kRhoExpHi = 139;
 
+// Bits of 2^23 in binary32: a position in [0, 2^23) plus 2^23, rounded toward
+// zero, has the bit pattern kTruncPattern + its integer part.
+constexpr uint32_t kTruncPattern = 0x4B000000u;
+
 // What a phantom's voxels hold, found on the device when the phantom is created
 // (which also packs each voxel's word): the first voxel whose material index is
 // out of range and the first whose density is neither 0 nor in [2^-18, 2^13) g/cm^3
@@ -157,7 +161,19 @@ int launch_scan_phantom(const uint8_t *mat, const float *rho, size_t nvox, int n
 struct SharedTables {
     int n_e, n_zeta, e_min;
     int max_n_mat;               // largest n_mat of the launch's requests (shared-memory size)
+    uint32_t cells;              // cells of one surface, (n_e - 1)(n_zeta - 1) mod 2^32
+    int wide;                    // some axis has more than 2^23 voxels or some cell index 2^32 or more (wide_index)
 };
+
+// Whether a request needs the general index arithmetic: positions are truncated
+// by an addition that holds up to 2^23 voxels per axis, and 32-bit cell indices
+// count fewer than 2^32 cells over the materials' surfaces.
+inline bool wide_index(int nx, int ny, int nz, int n_mat, int n_e, int n_zeta)
+{
+    const int lim = 1 << 23;
+    const double cells = static_cast<double>(n_mat) * (n_e - 1) * (n_zeta - 1);
+    return nx > lim || ny > lim || nz > lim || cells >= 4294967296.0;
+}
 
 struct LaunchParams {
     SharedTables sh;

@@ -297,7 +297,7 @@ enum { kEscaped = 0, kFictitious = 1, kReal = 2 };
 // attenuation table in shared memory.  An escape is counted by the caller,
 // outside the loop of flights, and the caller keeps ph.step below kMaxSteps
 // (the history's step limit).
-template <bool kKeys>
+template <bool kKeys, bool kWide>
 __device__ __forceinline__ int flight(const SharedTables &sh, const RequestDesc &q, const float4 *__restrict__ s_tab,
                                       Photon &ph, LaneCounts &cnt, Hit &hit)
 {
@@ -320,15 +320,23 @@ __device__ __forceinline__ int flight(const SharedTables &sh, const RequestDesc 
     if (!(__float_as_uint(fx) < __float_as_uint(q.fnx) && __float_as_uint(fy) < __float_as_uint(q.fny) &&
           __float_as_uint(fz) < __float_as_uint(q.fnz)))
         return kEscaped;
-    const uint32_t idx = static_cast<uint32_t>(static_cast<int>(fx)) +
-                         static_cast<uint32_t>(q.nx) *
-                             (static_cast<uint32_t>(static_cast<int>(fy)) +
-                              static_cast<uint32_t>(q.ny) * static_cast<uint32_t>(static_cast<int>(fz)));
-    // one gather: the material in the top 4 bits, the density's exponent rebased
+    uint32_t idx;
+    if (kWide) {
+        idx = static_cast<uint32_t>(static_cast<int>(fx)) +
+              static_cast<uint32_t>(q.nx) * (static_cast<uint32_t>(static_cast<int>(fy)) +
+                                             static_cast<uint32_t>(q.ny) * static_cast<uint32_t>(static_cast<int>(fz)));
+    } else {
+        // the integer parts from additions rounded toward zero; idx0 takes their
+        // exponent bits off (all modulo 2^32)
+        idx = __float_as_uint(trunc_up(fx)) + static_cast<uint32_t>(q.nx) * __float_as_uint(trunc_up(fy)) +
+              q.nxy * __float_as_uint(trunc_up(fz)) + q.idx0;
+    }
+    // one gather: the material in the top 4 bits, the density's exponent rebased.  The
+    // low 28 bits read as binary32 are the density times 2^-kRhoExpBias (0 for 0, else
+    // normal), so one exact multiplication restores it.
     const uint32_t w = __ldg(&q.vox[idx]);
     const int m = static_cast<int>(w >> 28);
-    const uint32_t rb = w & 0x0fffffffu;
-    const float rho = rb ? __uint_as_float(rb + (kRhoExpBias << 23)) : 0.0f;
+    const float rho = __uint_as_float(w & 0x0fffffffu) * kRhoScale;
     // interaction type with probabilities mu_i / mu_max: fictitious when u1 is at or
     // above the total share; otherwise the first cumulative share above u1.  The
     // table's fourth column is the total share's node difference, so a fictitious
@@ -358,7 +366,7 @@ __device__ __forceinline__ int flight(const SharedTables &sh, const RequestDesc 
 
 // A real interaction: local deposition, C/R-surface polar angle, rotation.
 // Returns false when the history has ended.
-template <bool kTrace>
+template <bool kWide, bool kTrace>
 __device__ __forceinline__ bool interact(const SharedTables &sh, const RequestDesc &q, const float *__restrict__ s_mm,
                                          Photon &ph, const Hit &hit, LaneCounts &cnt, const Tracer &tr)
 {
@@ -370,10 +378,17 @@ __device__ __forceinline__ bool interact(const SharedTables &sh, const RequestDe
         if (kTrace) tr.end(ph.h, kEndPe, ph.step, ph.e);
         return false;
     }
-    const float *S = hit.type == 1
-                         ? q.csurf + static_cast<size_t>(hit.m) * q.cs_stride * 4
-                         : q.rsurf + static_cast<size_t>(hit.m) * (sh.n_e - 1) * (sh.n_zeta - 1) * 4;
-    const float mu = surface(S, sh.n_zeta, ph.j, ph.te, uni(hit.rz));
+    const float *S = hit.type == 1 ? q.csurf : q.rsurf;
+    float mu;
+    if (kWide) {
+        const size_t cells = static_cast<size_t>(sh.n_e - 1) * (sh.n_zeta - 1);
+        const size_t first = hit.type == 1 && q.cs_stride == 0 ? 0 : hit.m * cells;
+        mu = surface(S, first + static_cast<size_t>(ph.j) * (sh.n_zeta - 1), sh.n_zeta, ph.te, uni(hit.rz));
+    } else {
+        const uint32_t stride = hit.type == 1 ? static_cast<uint32_t>(q.cs_stride) : sh.cells;
+        mu = surface(S, static_cast<uint32_t>(hit.m) * stride + static_cast<uint32_t>(ph.j) * (sh.n_zeta - 1), sh.n_zeta,
+                     ph.te, uni(hit.rz));
+    }
     if (hit.type == 1) {
         // Compton: E' = E / (1 + (E/mc^2)(1 - mu)), the electron gets E - E'
         cnt.event(kCntCompton);
@@ -427,7 +442,7 @@ static_assert(kWarpBytes % 16 == 0, "a warp's shared-memory area must keep 16-by
 
 // All histories [q.local_begin, q.local_end) of one request, claimed by warps
 // from q.work in runs of `chunk`.  Returns when the warp has no photon left.
-template <bool kKeys, bool kFluence, bool kTrace>
+template <bool kKeys, bool kFluence, bool kWide, bool kTrace>
 __device__ __forceinline__ void run_request(const LaunchParams &P, const RequestDesc &q, const float4 *s_tab,
                                             const float *s_mm, const Queue &Q, int lane, LaneCounts &cnt)
 {
@@ -538,7 +553,7 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
                 Hit hit;
                 int f, k = 0;
                 do {
-                    f = flight<kKeys>(P.sh, q, s_tab, ph, cnt, hit);
+                    f = flight<kKeys, kWide>(P.sh, q, s_tab, ph, cnt, hit);
                 } while (f == kFictitious && ++k < lim);
                 if (f == kEscaped) {
                     cnt.event(kCntEscaped);
@@ -546,7 +561,7 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
                     if (kTrace) tr.end(ph.h, kEndEscaped, ph.step, 0.0f);
                     alive = false;
                 } else if (f == kReal) {
-                    alive = interact<kTrace>(P.sh, q, s_mm, ph, hit, cnt, tr);
+                    alive = interact<kWide, kTrace>(P.sh, q, s_mm, ph, hit, cnt, tr);
                 }
             }
         }
@@ -576,7 +591,7 @@ __device__ __forceinline__ void load_tables(const RequestDesc &q, int n_e, float
 // kTrace (single-request forms): also write each history's record to P.trace.
 constexpr int kReqWords = sizeof(RequestDesc) / 16;
 
-template <int kMaxThreads, int kMinBlocks, int kForm, bool kTrace = false>
+template <int kMaxThreads, int kMinBlocks, int kForm, bool kWide, bool kTrace>
 __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(const LaunchParams P)
 {
     extern __shared__ float4 smem[];
@@ -602,7 +617,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
     if (!kMulti) {
         load_tables(P.one, n_e, s_tab, s_mm);
         __syncthreads();
-        run_request<true, kForm == 1, kTrace>(P, P.one, s_tab, s_mm, Q, lane, cnt);
+        run_request<true, kForm == 1, kWide, kTrace>(P, P.one, s_tab, s_mm, Q, lane, cnt);
         flush_warp(P.one.counts, cnt, lane);
         return;
     }
@@ -629,7 +644,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
         const float4 *src = reinterpret_cast<const float4 *>(P.reqs + found);
         for (int i = lane; i < kReqWords; i += 32) w_req4[i] = src[i];
         __syncwarp();
-        run_request<true, kForm == 3, false>(P, q, reinterpret_cast<const float4 *>(q.tab), q.mmax, Q, lane, cnt);
+        run_request<true, kForm == 3, kWide, false>(P, q, reinterpret_cast<const float4 *>(q.tab), q.mmax, Q, lane, cnt);
         flush_warp(q.counts, cnt, lane);
         __syncwarp();
         // the same request is exhausted now; continue the walk from it
@@ -645,7 +660,7 @@ __global__ void sample_mu_kernel(const float *surf, int n_zeta, int n_e, int e_m
     for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
         const U4 b = block(seed, i, 0, kStreamSampler);
-        out[i] = static_cast<double>(surface(surf, n_zeta, j, te, uni(b.x)));
+        out[i] = static_cast<double>(surface(surf, static_cast<size_t>(j) * (n_zeta - 1), n_zeta, te, uni(b.x)));
     }
 }
 
@@ -666,11 +681,11 @@ __global__ void eval_math_kernel(int fn, const float *x, float *out, size_t n)
     }
 }
 
-template <int kMaxThreads, int kMinBlocks, int kForm, bool kTrace = false>
+template <int kMaxThreads, int kMinBlocks, int kForm, bool kWide = false, bool kTrace = false>
 int launch_t(const LaunchParams &p, int grid, int block, size_t smem, cudaStream_t stream,
              const L2Window *win = nullptr)
 {
-    auto *k = transport_kernel<kMaxThreads, kMinBlocks, kForm, kTrace>;
+    auto *k = transport_kernel<kMaxThreads, kMinBlocks, kForm, kWide, kTrace>;
     if (smem > 48 * 1024) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
             return CTD_ECUDA;
@@ -737,9 +752,13 @@ int launch_transport(const LaunchParams &p, int grid, int block, int threads_per
             set_error("trace launches take one request");
             return CTD_EINVAL;
         }
-        return p.one.fl_n > 0 ? launch_t<256, 4, 1, true>(p, grid, block, smem, s)
-                              : launch_t<256, 4, 0, true>(p, grid, block, smem, s);
+        if (p.sh.wide) return launch_t<256, 3, 1, true, true>(p, grid, block, smem, s);
+        return p.one.fl_n > 0 ? launch_t<256, 4, 1, false, true>(p, grid, block, smem, s)
+                              : launch_t<256, 4, 0, false, true>(p, grid, block, smem, s);
     }
+    // general index arithmetic (wide_index): one instantiation per form, whatever the residency
+    if (p.sh.wide) return p.n_req > 0 ? launch_t<256, 3, 3, true>(p, grid, block, smem, s, win)
+                                      : launch_t<256, 3, 1, true>(p, grid, block, smem, s, win);
     if (p.n_req > 0) return p.any_fluence ? launch_m<3>(p, grid, block, threads_per_sm, smem, s, win)
                                            : launch_m<2>(p, grid, block, threads_per_sm, smem, s, win);
     return p.one.fl_n > 0 ? launch_m<1>(p, grid, block, threads_per_sm, smem, s, win)
