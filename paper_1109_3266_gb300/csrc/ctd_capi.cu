@@ -163,7 +163,16 @@ int build_tables(ctd_ctx *ctx, Phantom &P)
     if ((rc = P.tab.ensure(P.h_tab.size())) || (rc = P.mm.ensure(n_e)) || (rc = P.cs.ensure(cs_cells.size())) ||
         (rc = P.rs.ensure(rs_cells.size())))
         return rc;
-    CK(cudaMemcpyAsync(P.tab.p, P.h_tab.data(), P.h_tab.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    // on the device the two columns every step reads (total share, its difference) and
+    // the two only a real interaction reads lie in separate planes
+    std::vector<float> planes(P.h_tab.size());
+    for (size_t i = 0, n = P.h_tab.size() / 4; i < n; ++i) {
+        planes[2 * i] = P.h_tab[4 * i + 2];
+        planes[2 * i + 1] = P.h_tab[4 * i + 3];
+        planes[2 * (n + i)] = P.h_tab[4 * i];
+        planes[2 * (n + i) + 1] = P.h_tab[4 * i + 1];
+    }
+    CK(cudaMemcpyAsync(P.tab.p, planes.data(), planes.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(P.mm.p, P.h_mm.data(), n_e * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(P.cs.p, cs_cells.data(), cs_cells.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(P.rs.p, rs_cells.data(), rs_cells.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));

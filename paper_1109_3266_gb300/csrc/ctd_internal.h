@@ -90,7 +90,7 @@ enum { kCntPe = 0, kCntCompton, kCntRayleigh, kCntFict, kCntEscaped, kCntMissed,
 struct alignas(16) RequestDesc {
     const uint32_t *vox;         // [nvox] material and density of each voxel, one word (kRhoExpBias)
     uint32_t nxy, idx0;          // nx * ny and -kTruncBits (1 + nx + nxy) mod 2^32 (the voxel index from truncated positions)
-    const float *tab;            // [n_mat][n_e][4]: c1, c2, c3 (cm^2/g), c3[j+1] - c3[j] in binary32
+    const float *tab;            // [n_mat][n_e][2]: c3 (cm^2/g), c3[j+1] - c3[j] in binary32; then [n_mat][n_e][2]: c1, c2
     const float *mmax;           // [n_e] majorant mu_max(E), 1/cm
     // R and C surfaces as cells of 4 floats, [n_e - 1][n_zeta - 1] per surface: cell (j, i)
     // holds S[j][i], S[j][i+1], S[j+1][i], S[j+1][i+1], the corners of one bilinear lookup

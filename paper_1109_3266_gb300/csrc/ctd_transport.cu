@@ -52,48 +52,43 @@ __device__ __forceinline__ void set_energy(Photon &ph, const SharedTables &sh, c
     ph.imax = 1.0f / __fmaf_rn(ph.te, m1 - m0, m0);
 }
 
-// A lane's once-per-history event counts, energy totals and the real
-// interactions of its current photon, in shared memory: they change at most a
-// few times per history, and registers are what bounds the kernel's residency.
+// How a photon's flight through the phantom ends, as counted by a lane; misses are
+// the source photons that end in none of these.
+enum { kNotEnded = -1, kDonePe, kDoneCutoff, kDoneEscaped, kDoneTerminated, kDoneAborted, kDoneKinds };
+
+// A lane's counts of ended histories, energy totals and the real interactions of
+// its current photon, in shared memory: they change at most a few times per
+// history, and registers are what bounds the kernel's residency.
 struct LaneSlot {
     unsigned long long e_emitted, e_escaped;   // keV * 2^23
-    uint32_t ev[6];                            // PE, escaped, missed, cutoff, terminated, aborted
+    uint32_t done[kDoneKinds];
     uint32_t nreal;                            // real interactions of the current photon
-    uint32_t pad;
 };
-static_assert(sizeof(LaneSlot) == 48, "LaneSlot layout");
+static_assert(sizeof(LaneSlot) == 40, "LaneSlot layout");
 
-// Event counts of a lane: the per-step events (fictitious, Compton, Rayleigh)
-// in registers, the rest in the lane's slot.  Woodcock steps are not counted:
-// each ends in exactly one of escape, fictitious, PE, Compton or Rayleigh.
+// Event counts of a lane: scatters and the Woodcock steps of ended histories in
+// registers, the rest in the lane's slot.  Fictitious events are not counted: each
+// step ends in exactly one of escape, fictitious, PE, Compton or Rayleigh.
 struct LaneCounts {
-    uint32_t fict, compton, rayleigh;
+    uint32_t steps, compton, rayleigh;
     LaneSlot *me;
     __device__ __forceinline__ void clear()
     {
-        fict = compton = rayleigh = 0;
+        steps = compton = rayleigh = 0;
         me->e_emitted = 0;
         me->e_escaped = 0;
 #pragma unroll
-        for (int i = 0; i < 6; ++i) me->ev[i] = 0;
-    }
-    // k is a constant at every call site, so the switch folds away
-    __device__ __forceinline__ void event(int k)
-    {
-        switch (k) {
-        case kCntFict: ++fict; break;
-        case kCntCompton: ++compton; break;
-        case kCntRayleigh: ++rayleigh; break;
-        case kCntPe: ++me->ev[0]; break;
-        case kCntEscaped: ++me->ev[1]; break;
-        case kCntMissed: ++me->ev[2]; break;
-        case kCntCutoff: ++me->ev[3]; break;
-        case kCntTerminated: ++me->ev[4]; break;
-        default: ++me->ev[5]; break;   // kCntAborted
-        }
+        for (int i = 0; i < kDoneKinds; ++i) me->done[i] = 0;
     }
     __device__ __forceinline__ void emitted(float e) { me->e_emitted += kev_fixed(e); }
-    __device__ __forceinline__ void escaped(float e) { me->e_escaped += kev_fixed(e); }
+    // the history ended after n steps with energy e left (counted as escaped unless
+    // the last event deposited it)
+    __device__ __forceinline__ void end(int how, uint32_t n, float e)
+    {
+        ++me->done[how];
+        steps += n;
+        if (how >= kDoneEscaped) me->e_escaped += kev_fixed(e);
+    }
 };
 
 // Per-history records of a trace launch (kTrace instantiations only): each
@@ -123,36 +118,37 @@ struct Tracer {
 };
 
 // A warp's counts added to a request's totals: warp sums, one atomic per
-// counter (energies as 128-bit fixed-point totals).  Leaves the counts cleared.
-__device__ __forceinline__ void flush_warp(DeviceCounts *dst, LaneCounts &c, int lane)
+// counter (energies as 128-bit fixed-point totals).  `sourced` is the warp's number
+// of source photons.  Leaves the counts cleared.
+__device__ __forceinline__ void flush_warp(DeviceCounts *dst, LaneCounts &c, uint64_t sourced, int lane)
 {
     __syncwarp();
     const LaneSlot &m = *c.me;
-    uint32_t v[10];
-    v[kCntPe] = m.ev[0];
-    v[kCntCompton] = c.compton;
-    v[kCntRayleigh] = c.rayleigh;
-    v[kCntFict] = c.fict;
-    v[kCntEscaped] = m.ev[1];
-    v[kCntMissed] = m.ev[2];
-    v[kCntCutoff] = m.ev[3];
-    v[kCntTerminated] = m.ev[4];
-    v[kCntAborted] = m.ev[5];
-    v[kCntSteps] = m.ev[1] + c.fict + m.ev[0] + c.compton + c.rayleigh;
-#pragma unroll
-    for (int i = 0; i < 10; ++i) {
-        unsigned long long x = v[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
-        if (lane == 0 && x) atomicAdd(&dst->n[i], x);
-    }
+    unsigned long long v[kDoneKinds + 3] = {m.done[kDonePe],         m.done[kDoneCutoff],  m.done[kDoneEscaped],
+                                            m.done[kDoneTerminated], m.done[kDoneAborted], c.steps,
+                                            c.compton,               c.rayleigh};
     unsigned long long em = m.e_emitted, es = m.e_escaped;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int i = 0; i < kDoneKinds + 3; ++i) v[i] += __shfl_down_sync(kFull, v[i], o);
         em += __shfl_down_sync(kFull, em, o);
         es += __shfl_down_sync(kFull, es, o);
     }
-    if (lane == 0) {
+    if (lane == 0 && sourced) {
+        const unsigned long long steps = v[kDoneKinds], compton = v[kDoneKinds + 1], rayleigh = v[kDoneKinds + 2];
+        const unsigned long long ended =
+            v[kDonePe] + v[kDoneCutoff] + v[kDoneEscaped] + v[kDoneTerminated] + v[kDoneAborted];
+        atomicAdd(&dst->n[kCntPe], v[kDonePe]);
+        atomicAdd(&dst->n[kCntCompton], compton);
+        atomicAdd(&dst->n[kCntRayleigh], rayleigh);
+        atomicAdd(&dst->n[kCntFict], steps - v[kDonePe] - v[kDoneEscaped] - compton - rayleigh);
+        atomicAdd(&dst->n[kCntEscaped], v[kDoneEscaped]);
+        atomicAdd(&dst->n[kCntMissed], sourced - ended);
+        atomicAdd(&dst->n[kCntCutoff], v[kDoneCutoff]);
+        atomicAdd(&dst->n[kCntTerminated], v[kDoneTerminated]);
+        atomicAdd(&dst->n[kCntAborted], v[kDoneAborted]);
+        atomicAdd(&dst->n[kCntSteps], steps);
         const unsigned long long o1 = atomicAdd(&dst->e_fix[0], em);
         if (o1 + em < o1) atomicAdd(&dst->e_fix[1], 1ull);
         const unsigned long long o2 = atomicAdd(&dst->e_fix[2], es);
@@ -231,8 +227,7 @@ __device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, uint64_
         }
     }
     if (!accepted) {
-        cnt.event(kCntAborted);
-        cnt.escaped(e);
+        cnt.end(kDoneAborted, 0, e);
         if (kTrace) tr.end(h, kEndAborted, 0, 0.0f);
         return false;
     }
@@ -263,8 +258,7 @@ __device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, uint64_
     float tn = fmaxf(fmaxf(fminf(t0x, t1x), fminf(t0y, t1y)), fminf(t0z, t1z));
     const float tf = fminf(fminf(fmaxf(t0x, t1x), fmaxf(t0y, t1y)), fmaxf(t0z, t1z));
     if (!(tn < tf) || !(tf > 0.0f)) {
-        cnt.event(kCntMissed);
-        cnt.escaped(e);
+        cnt.me->e_escaped += kev_fixed(e);
         if (kTrace) tr.end(h, kEndMissed, 0, 0.0f);
         return false;
     }
@@ -282,31 +276,35 @@ __device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, uint64_
     return true;
 }
 
-// Site of a real interaction found by a flight
-struct Hit {
-    uint32_t idx;     // voxel (phantoms hold fewer than 2^32 voxels)
+// Where a flight ended and the numbers its interaction needs
+struct Site {
+    bool inside, fictitious;
+    uint32_t idx;     // voxel (phantoms hold fewer than 2^32 voxels; 0 outside the phantom)
     int m;            // material
-    int type;         // 0 photoelectric, 1 Compton, 2 Rayleigh
+    float y, sr;      // u1 and rho / mu_max
     uint32_t rz, rw;  // the step's random words for zeta and phi
 };
 
-enum { kEscaped = 0, kFictitious = 1, kReal = 2 };
-
 // One Woodcock flight (Sec. 2.1): free path against mu_max(E), the move, the
-// escape test, the voxel and the interaction type.  s_tab is the request's
-// attenuation table in shared memory.  An escape is counted by the caller,
-// outside the loop of flights, and the caller keeps ph.step below kMaxSteps
-// (the history's step limit).
+// escape test, the voxel and whether its interaction is fictitious.  s_tab is the
+// request's attenuation table.  The caller keeps ph.step below kMaxSteps (the
+// history's step limit).
+//
+// A flight and an interaction are bound by the latency of their own instruction
+// chains at eight warps per scheduler (ncu: issue active 75 %, of a warp's ten
+// cycles per instruction 2.4 wait on the previous one, 0.6 on a branch), so each is
+// one basic block: a photon that left the phantom looks voxel 0 up and discards
+// it, all interaction types take the same path, and the compiler fills one
+// chain's waits with another's instructions.  With a branch per outcome CBCT water
+// took 16.70 ms of transport per 2e8 histories and the head 28.43; without,
+// 15.31 and 25.03 ms (bit-identical).
 template <bool kKeys, bool kWide>
-__device__ __forceinline__ int flight(const SharedTables &sh, const RequestDesc &q, const float4 *__restrict__ s_tab,
-                                      Photon &ph, LaneCounts &cnt, Hit &hit)
+__device__ __forceinline__ void flight(const SharedTables &sh, const RequestDesc &q, const float2 *__restrict__ s_tab,
+                                       Photon &ph, Site &at)
 {
     const U4 b = draw<kKeys>(q, ph.h, ph.step, kStreamTransport);
     ph.step++;
-    const int n_e = sh.n_e;
-    const int j = ph.j;
-    const float te = ph.te, imax = ph.imax;
-    const float path = (-log32(uni(b.x))) * imax;
+    const float path = (-log32(uni(b.x))) * ph.imax;
     // the move in voxel units: each displacement s u_k times 1/d_k, added fused
     ph.x = __fmaf_rn(path * ph.ux, q.ix, ph.x);
     ph.y = __fmaf_rn(path * ph.uy, q.iy, ph.y);
@@ -317,123 +315,124 @@ __device__ __forceinline__ int flight(const SharedTables &sh, const RequestDesc 
     // sign bit or an all-ones exponent, so larger patterns than n), and a position
     // is never -0 (the entry point is clamped to +0 at least, and adding a nonzero
     // or +0 displacement to a value other than -0 never gives -0)
-    if (!(__float_as_uint(fx) < __float_as_uint(q.fnx) && __float_as_uint(fy) < __float_as_uint(q.fny) &&
-          __float_as_uint(fz) < __float_as_uint(q.fnz)))
-        return kEscaped;
+    at.inside = __float_as_uint(fx) < __float_as_uint(q.fnx) && __float_as_uint(fy) < __float_as_uint(q.fny) &&
+                __float_as_uint(fz) < __float_as_uint(q.fnz);
     uint32_t idx;
     if (kWide) {
-        idx = static_cast<uint32_t>(static_cast<int>(fx)) +
-              static_cast<uint32_t>(q.nx) * (static_cast<uint32_t>(static_cast<int>(fy)) +
-                                             static_cast<uint32_t>(q.ny) * static_cast<uint32_t>(static_cast<int>(fz)));
+        idx = at.inside ? static_cast<uint32_t>(static_cast<int>(fx)) +
+                              static_cast<uint32_t>(q.nx) *
+                                  (static_cast<uint32_t>(static_cast<int>(fy)) +
+                                   static_cast<uint32_t>(q.ny) * static_cast<uint32_t>(static_cast<int>(fz)))
+                        : 0u;
     } else {
         // the integer parts from additions rounded toward zero; idx0 takes their
         // exponent bits off (all modulo 2^32)
         idx = __float_as_uint(trunc_up(fx)) + static_cast<uint32_t>(q.nx) * __float_as_uint(trunc_up(fy)) +
               q.nxy * __float_as_uint(trunc_up(fz)) + q.idx0;
+        idx = at.inside ? idx : 0u;
     }
     // one gather: the material in the top 4 bits, the density's exponent rebased.  The
     // low 28 bits read as binary32 are the density times 2^-kRhoExpBias (0 for 0, else
     // normal), so one exact multiplication restores it.
     const uint32_t w = __ldg(&q.vox[idx]);
-    const int m = static_cast<int>(w >> 28);
+    at.idx = idx;
+    at.m = static_cast<int>(w >> 28);
     const float rho = __uint_as_float(w & 0x0fffffffu) * kRhoScale;
     // interaction type with probabilities mu_i / mu_max: fictitious when u1 is at or
-    // above the total share; otherwise the first cumulative share above u1.  The
-    // table's fourth column is the total share's node difference, so a fictitious
-    // step reads one node; a real one reads the next node's c1 and c2 as well.
-    const float4 A = s_tab[m * n_e + j];
-    const float y = uni(b.y);
-    const float sr = rho * imax;
-    const float c3 = __fmaf_rn(te, A.w, A.z);
-    if (!(y < sr * c3)) {
-        cnt.event(kCntFict);
-        return kFictitious;
-    }
-    const float2 B = *reinterpret_cast<const float2 *>(&s_tab[m * n_e + j + 1]);
-    const float c1 = __fmaf_rn(te, B.x - A.x, A.x);
-    const float c2 = __fmaf_rn(te, B.y - A.y, A.y);
-    int type;
-    if (y < sr * c1) type = 0;
-    else if (y < sr * c2) type = 1;
-    else type = 2;
-    hit.idx = idx;
-    hit.m = m;
-    hit.type = type;
-    hit.rz = b.z;
-    hit.rw = b.w;
-    return kReal;
+    // above the total share.  The table's first plane holds the total share and its
+    // difference to the next node.
+    const float2 T = s_tab[at.m * sh.n_e + ph.j];
+    at.y = uni(b.y);
+    at.sr = rho * ph.imax;
+    at.fictitious = at.inside && !(at.y < at.sr * __fmaf_rn(ph.te, T.y, T.x));
+    at.rz = b.z;
+    at.rw = b.w;
 }
 
-// A real interaction: local deposition, C/R-surface polar angle, rotation.
-// Returns false when the history has ended.
-template <bool kWide, bool kTrace>
-__device__ __forceinline__ bool interact(const SharedTables &sh, const RequestDesc &q, const float *__restrict__ s_mm,
-                                         Photon &ph, const Hit &hit, LaneCounts &cnt, const Tracer &tr)
+// A real interaction: the type (the first cumulative share above u1, from c1 and c2
+// of both nodes in the table's second plane), the C/R-surface polar angle, local
+// deposition, rotation.  Returns how the history ended, or kNotEnded.  Straight-line
+// code for all types (see flight): a Rayleigh event is a scatter with E' = E (which
+// deposits 0 and leaves node and majorant as they were), and an absorbed photon's
+// angle is discarded.  kAnyMode: the request may limit the real interactions
+// (CTD_MODE_MAX_REAL), where most histories end here and skip the rest; full
+// transport is compiled without that branch (with it 2 % slower on CBCT water, while
+// a primary-only run without it was 4 % slower).
+template <bool kWide, bool kAnyMode, bool kTrace>
+__device__ __forceinline__ int interact(const SharedTables &sh, const RequestDesc &q, const float2 *__restrict__ s_tab,
+                                        const float *__restrict__ s_mm, Photon &ph, const Site &at, LaneCounts &cnt,
+                                        const Tracer &tr)
 {
-    if (kTrace) tr.last(ph.h, hit.type, hit.idx);
-    if (hit.type == 0) {
-        // photoelectric absorption: the electron deposits E here
-        cnt.event(kCntPe);
-        deposit(q.tally, hit.idx, ph.e);
-        if (kTrace) tr.end(ph.h, kEndPe, ph.step, ph.e);
-        return false;
-    }
-    const float *S = hit.type == 1 ? q.csurf : q.rsurf;
+    const float2 *t = s_tab + ((q.n_mat + at.m) * sh.n_e + ph.j);
+    const float2 A = t[0], B = t[1];
+    const float c1 = __fmaf_rn(ph.te, B.x - A.x, A.x);
+    const float c2 = __fmaf_rn(ph.te, B.y - A.y, A.y);
+    const bool pe = at.y < at.sr * c1;
+    const bool compton = !pe && at.y < at.sr * c2;
+    const bool rayleigh = !pe && !compton;
+    const float *S = rayleigh ? q.rsurf : q.csurf;
     float mu;
     if (kWide) {
         const size_t cells = static_cast<size_t>(sh.n_e - 1) * (sh.n_zeta - 1);
-        const size_t first = hit.type == 1 && q.cs_stride == 0 ? 0 : hit.m * cells;
-        mu = surface(S, first + static_cast<size_t>(ph.j) * (sh.n_zeta - 1), sh.n_zeta, ph.te, uni(hit.rz));
+        const size_t first = !rayleigh && q.cs_stride == 0 ? 0 : at.m * cells;
+        mu = surface(S, first + static_cast<size_t>(ph.j) * (sh.n_zeta - 1), sh.n_zeta, ph.te, uni(at.rz));
     } else {
-        const uint32_t stride = hit.type == 1 ? static_cast<uint32_t>(q.cs_stride) : sh.cells;
-        mu = surface(S, static_cast<uint32_t>(hit.m) * stride + static_cast<uint32_t>(ph.j) * (sh.n_zeta - 1), sh.n_zeta,
-                     ph.te, uni(hit.rz));
+        const uint32_t stride = rayleigh ? sh.cells : static_cast<uint32_t>(q.cs_stride);
+        mu = surface(S, static_cast<uint32_t>(at.m) * stride + static_cast<uint32_t>(ph.j) * (sh.n_zeta - 1), sh.n_zeta,
+                     ph.te, uni(at.rz));
     }
-    if (hit.type == 1) {
-        // Compton: E' = E / (1 + (E/mc^2)(1 - mu)), the electron gets E - E'
-        cnt.event(kCntCompton);
-        const float k = ph.e * static_cast<float>(1.0 / kMec2);
-        const float ep = ph.e / __fmaf_rn(k, 1.0f - mu, 1.0f);
-        if (ep < static_cast<float>(sh.e_min)) {
-            cnt.event(kCntCutoff);
-            deposit(q.tally, hit.idx, ph.e);
-            if (kTrace) tr.end(ph.h, kEndCutoff, ph.step, ph.e);
-            return false;
-        }
-        deposit(q.tally, hit.idx, ph.e - ep);
-        if (kTrace) tr.end(ph.h, kEndTerminated, ph.step, ph.e - ep);   // kept if the history ends here
-        ph.e = ep;
+    // Compton: E' = E / (1 + (E/mc^2)(1 - mu)), the electron gets E - E' (all of E
+    // when E' is below the absorption energy); photoelectric absorption: all of E
+    const float e = ph.e;
+    const float k = e * static_cast<float>(1.0 / kMec2);
+    const float ec = e / __fmaf_rn(k, 1.0f - mu, 1.0f);
+    const bool cutoff = compton && ec < static_cast<float>(sh.e_min);
+    const bool absorbed = pe || cutoff;
+    ph.e = compton && !cutoff ? ec : e;
+    const float dep = absorbed ? e : e - ph.e;
+    deposit(q.tally, at.idx, dep);
+    cnt.compton += compton;
+    cnt.rayleigh += rayleigh;
+    int end = pe ? kDonePe : cutoff ? kDoneCutoff : kNotEnded;
+    if (kAnyMode && q.mode == CTD_MODE_MAX_REAL && !absorbed && ++cnt.me->nreal >= static_cast<uint32_t>(q.max_real))
+        end = kDoneTerminated;
+    // (full transport takes no branch around a scatter's end: an absorbed photon's is
+    // discarded)
+    if (!kAnyMode || q.mode == CTD_MODE_FULL || end == kNotEnded) {
         set_energy(ph, sh, s_mm);
-    } else {
-        cnt.event(kCntRayleigh);
-        if (kTrace) tr.end(ph.h, kEndTerminated, ph.step, 0.0f);
+        rotate(ph.ux, ph.uy, ph.uz, mu, uni(at.rw));
     }
-    if (q.mode == CTD_MODE_MAX_REAL && ++cnt.me->nreal >= static_cast<uint32_t>(q.max_real)) {
-        cnt.event(kCntTerminated);
-        cnt.escaped(ph.e);
-        return false;
+    if (kTrace) {
+        tr.last(ph.h, pe ? 0 : compton ? 1 : 2, at.idx);
+        if (end != kNotEnded)
+            tr.end(ph.h, pe ? kEndPe : cutoff ? kEndCutoff : kEndTerminated, ph.step, dep);
     }
-    rotate(ph.ux, ph.uy, ph.uz, mu, uni(hit.rw));
-    return true;
+    return end;
 }
 
 // Per-warp photon queue in shared memory: source photons are made 32 at a
 // time by the whole warp and taken by lanes whose history has ended.
-constexpr int kQueue = 64;
-constexpr size_t kQueueBytes = kQueue * (7 * sizeof(float) + sizeof(uint64_t));
+constexpr int kQueue = 48, kQueueLow = 16;
+constexpr size_t kQueueBytes = kQueue * (2 * sizeof(float4) + sizeof(uint64_t));
 
-// A warp's claim of local history indices [next, end) and the 1 keV interval
-// of its first history, kept in shared memory (read only when the queue is
-// topped up).
+// A warp's claim of local history indices [next, end), the 1 keV interval of its
+// first history and the source photons the warp has made, kept in shared memory
+// (read only when the queue is topped up).
 struct WarpPool {
-    uint64_t next, end;
+    uint64_t next, end, sourced;
     int bin;
-    int pad[3];
+    int pad;
 };
 
+// Photons in vectors, so that one is stored or taken with three wide accesses; the
+// inverse majorant is worked out by the whole warp that made the photon.  Topped up
+// below 16 photons: 47 at most, and the tables, queues and slots of 32 warps leave
+// L1 more than 60 KB (with 28 KB, the largest shared-memory carve-out, CBCT water
+// took 9 % longer: the gathers' lines in flight need it).
 struct Queue {
-    uint64_t *h;
-    float *f;   // [7][kQueue]: x y z (voxel units) ux uy uz e
+    float4 *a;     // [kQueue] x, y, z (voxel units), ux
+    float4 *b;     // [kQueue] uy, uz, e, 1 / mu_max(e)
+    uint64_t *h;   // [kQueue]
     WarpPool *pool;
 };
 
@@ -442,8 +441,8 @@ static_assert(kWarpBytes % 16 == 0, "a warp's shared-memory area must keep 16-by
 
 // All histories [q.local_begin, q.local_end) of one request, claimed by warps
 // from q.work in runs of `chunk`.  Returns when the warp has no photon left.
-template <bool kKeys, bool kFluence, bool kWide, bool kTrace>
-__device__ __forceinline__ void run_request(const LaunchParams &P, const RequestDesc &q, const float4 *s_tab,
+template <bool kKeys, bool kFluence, bool kWide, bool kAnyMode, bool kTrace>
+__device__ __forceinline__ void run_request(const LaunchParams &P, const RequestDesc &q, const float2 *s_tab,
                                             const float *s_mm, const Queue &Q, int lane, LaneCounts &cnt)
 {
     Tracer tr;
@@ -458,12 +457,13 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
     if (lane == 0) {
         Q.pool->next = 0;
         Q.pool->end = 0;
+        Q.pool->sourced = 0;
         Q.pool->bin = 0;
     }
     __syncwarp();
     for (;;) {
         // top the queue up with one round of up to 32 source photons
-        if (qcount < 32 && !drained) {
+        if (qcount < kQueueLow && !drained) {
             uint64_t pool_next = Q.pool->next, pool_end = Q.pool->end;
             int pool_bin = Q.pool->bin;
             if (pool_next >= pool_end) {
@@ -491,17 +491,14 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
                 const unsigned okm = __ballot_sync(kFull, ok);
                 if (ok) {
                     const int slot = qcount + __popc(okm & lt_mask);
+                    set_energy(np, P.sh, s_mm);
+                    Q.a[slot] = make_float4(np.x, np.y, np.z, np.ux);
+                    Q.b[slot] = make_float4(np.uy, np.uz, np.e, np.imax);
                     Q.h[slot] = np.h;
-                    Q.f[0 * kQueue + slot] = np.x;
-                    Q.f[1 * kQueue + slot] = np.y;
-                    Q.f[2 * kQueue + slot] = np.z;
-                    Q.f[3 * kQueue + slot] = np.ux;
-                    Q.f[4 * kQueue + slot] = np.uy;
-                    Q.f[5 * kQueue + slot] = np.uz;
-                    Q.f[6 * kQueue + slot] = np.e;
                 }
                 qcount += __popc(okm);
                 pool_next += take;
+                if (lane == 0) Q.pool->sourced += take;
             }
             __syncwarp();
             if (lane == 0) {
@@ -518,17 +515,19 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
             const int rank = __popc(need & lt_mask);
             if (rank < npop) {
                 const int slot = qcount - 1 - rank;
+                const float4 a = Q.a[slot], b = Q.b[slot];
+                ph.x = a.x;
+                ph.y = a.y;
+                ph.z = a.z;
+                ph.ux = a.w;
+                ph.uy = b.x;
+                ph.uz = b.y;
+                ph.e = b.z;
+                ph.imax = b.w;
                 ph.h = Q.h[slot];
-                ph.x = Q.f[0 * kQueue + slot];
-                ph.y = Q.f[1 * kQueue + slot];
-                ph.z = Q.f[2 * kQueue + slot];
-                ph.ux = Q.f[3 * kQueue + slot];
-                ph.uy = Q.f[4 * kQueue + slot];
-                ph.uz = Q.f[5 * kQueue + slot];
-                ph.e = Q.f[6 * kQueue + slot];
+                ph.j = enode(ph.e, P.sh.e_min, P.sh.n_e, ph.te);
                 ph.step = 0;
-                cnt.me->nreal = 0;
-                set_energy(ph, P.sh, s_mm);
+                if (kAnyMode) cnt.me->nreal = 0;
                 alive = true;
             }
         }
@@ -542,32 +541,34 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
             // flights until a real interaction, the escape or flight_cap flights; then the
             // interaction.  A run stops short of the history's step limit; a history that
             // has reached it is aborted when its next run would start.
-            const uint32_t room = kMaxSteps - ph.step;
-            const int lim = room < static_cast<uint32_t>(P.flight_cap) ? static_cast<int>(room) : P.flight_cap;
+            int lim = P.flight_cap, end = kNotEnded;
+            if (ph.step + static_cast<uint32_t>(P.flight_cap) > kMaxSteps) lim = static_cast<int>(kMaxSteps - ph.step);
             if (lim == 0) {
-                cnt.event(kCntAborted);
-                cnt.escaped(ph.e);
+                end = kDoneAborted;
                 if (kTrace) tr.end(ph.h, kEndAborted, ph.step, 0.0f);
-                alive = false;
             } else {
-                Hit hit;
-                int f, k = 0;
+                Site at;
+                int k = 0;
                 do {
-                    f = flight<kKeys, kWide>(P.sh, q, s_tab, ph, cnt, hit);
-                } while (f == kFictitious && ++k < lim);
-                if (f == kEscaped) {
-                    cnt.event(kCntEscaped);
-                    cnt.escaped(ph.e);
+                    flight<kKeys, kWide>(P.sh, q, s_tab, ph, at);
+                } while (at.fictitious && ++k < lim);
+                if (!at.inside) {
+                    end = kDoneEscaped;
                     if (kTrace) tr.end(ph.h, kEndEscaped, ph.step, 0.0f);
-                    alive = false;
-                } else if (f == kReal) {
-                    alive = interact<kWide, kTrace>(P.sh, q, s_mm, ph, hit, cnt, tr);
+                } else if (!at.fictitious) {
+                    end = interact<kWide, kAnyMode, kTrace>(P.sh, q, s_tab, s_mm, ph, at, cnt, tr);
                 }
+            }
+            // every way a history ends meets here, so that its lanes are counted together
+            if (end != kNotEnded) {
+                cnt.end(end, ph.step, ph.e);
+                alive = false;
             }
         }
     }
 }
 
+// the two table planes are 16 n_mat n_e bytes in all
 __device__ __forceinline__ void load_tables(const RequestDesc &q, int n_e, float4 *s_tab, float *s_mm)
 {
     const int ntab = q.n_mat * n_e;
@@ -591,7 +592,7 @@ __device__ __forceinline__ void load_tables(const RequestDesc &q, int n_e, float
 // kTrace (single-request forms): also write each history's record to P.trace.
 constexpr int kReqWords = sizeof(RequestDesc) / 16;
 
-template <int kMaxThreads, int kMinBlocks, int kForm, bool kWide, bool kTrace>
+template <int kMaxThreads, int kMinBlocks, int kForm, bool kWide, bool kAnyMode, bool kTrace>
 __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(const LaunchParams P)
 {
     extern __shared__ float4 smem[];
@@ -607,8 +608,9 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
                                   : reinterpret_cast<unsigned char *>(smem + P.sh.max_n_mat * n_e + (n_e + 3) / 4) +
                                         warp * kWarpBytes;
     Queue Q;
-    Q.h = reinterpret_cast<uint64_t *>(wbase);
-    Q.f = reinterpret_cast<float *>(Q.h + kQueue);
+    Q.a = reinterpret_cast<float4 *>(wbase);
+    Q.b = Q.a + kQueue;
+    Q.h = reinterpret_cast<uint64_t *>(Q.b + kQueue);
     Q.pool = reinterpret_cast<WarpPool *>(wbase + kQueueBytes);
     LaneCounts cnt;
     cnt.me = reinterpret_cast<LaneSlot *>(wbase + kQueueBytes + sizeof(WarpPool)) + lane;
@@ -617,8 +619,8 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
     if (!kMulti) {
         load_tables(P.one, n_e, s_tab, s_mm);
         __syncthreads();
-        run_request<true, kForm == 1, kWide, kTrace>(P, P.one, s_tab, s_mm, Q, lane, cnt);
-        flush_warp(P.one.counts, cnt, lane);
+        run_request<true, kForm == 1, kWide, kAnyMode, kTrace>(P, P.one, reinterpret_cast<const float2 *>(s_tab), s_mm, Q, lane, cnt);
+        flush_warp(P.one.counts, cnt, Q.pool->sourced, lane);
         return;
     }
     // every warp starts at the first request and walks forward to the next request
@@ -644,8 +646,8 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
         const float4 *src = reinterpret_cast<const float4 *>(P.reqs + found);
         for (int i = lane; i < kReqWords; i += 32) w_req4[i] = src[i];
         __syncwarp();
-        run_request<true, kForm == 3, kWide, false>(P, q, reinterpret_cast<const float4 *>(q.tab), q.mmax, Q, lane, cnt);
-        flush_warp(q.counts, cnt, lane);
+        run_request<true, kForm == 3, kWide, true, false>(P, q, reinterpret_cast<const float2 *>(q.tab), q.mmax, Q, lane, cnt);
+        flush_warp(q.counts, cnt, Q.pool->sourced, lane);
         __syncwarp();
         // the same request is exhausted now; continue the walk from it
         r = found;
@@ -681,11 +683,11 @@ __global__ void eval_math_kernel(int fn, const float *x, float *out, size_t n)
     }
 }
 
-template <int kMaxThreads, int kMinBlocks, int kForm, bool kWide = false, bool kTrace = false>
+template <int kMaxThreads, int kMinBlocks, int kForm, bool kWide = false, bool kAnyMode = false, bool kTrace = false>
 int launch_t(const LaunchParams &p, int grid, int block, size_t smem, cudaStream_t stream,
              const L2Window *win = nullptr)
 {
-    auto *k = transport_kernel<kMaxThreads, kMinBlocks, kForm, kWide, kTrace>;
+    auto *k = transport_kernel<kMaxThreads, kMinBlocks, kForm, kWide, kAnyMode, kTrace>;
     if (smem > 48 * 1024) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
             return CTD_ECUDA;
@@ -752,13 +754,17 @@ int launch_transport(const LaunchParams &p, int grid, int block, int threads_per
             set_error("trace launches take one request");
             return CTD_EINVAL;
         }
-        if (p.sh.wide) return launch_t<256, 3, 1, true, true>(p, grid, block, smem, s);
-        return p.one.fl_n > 0 ? launch_t<256, 4, 1, false, true>(p, grid, block, smem, s)
-                              : launch_t<256, 4, 0, false, true>(p, grid, block, smem, s);
+        if (p.sh.wide) return launch_t<256, 3, 1, true, true, true>(p, grid, block, smem, s);
+        return p.one.fl_n > 0 ? launch_t<256, 4, 1, false, true, true>(p, grid, block, smem, s)
+                              : launch_t<256, 4, 0, false, true, true>(p, grid, block, smem, s);
     }
     // general index arithmetic (wide_index): one instantiation per form, whatever the residency
-    if (p.sh.wide) return p.n_req > 0 ? launch_t<256, 3, 3, true>(p, grid, block, smem, s, win)
-                                      : launch_t<256, 3, 1, true>(p, grid, block, smem, s, win);
+    if (p.sh.wide) return p.n_req > 0 ? launch_t<256, 3, 3, true, true>(p, grid, block, smem, s, win)
+                                      : launch_t<256, 3, 1, true, true>(p, grid, block, smem, s, win);
+    // a limit on real interactions: likewise (64 registers suit every residency; interact)
+    if (p.n_req == 0 && p.one.mode != CTD_MODE_FULL)
+        return p.one.fl_n > 0 ? launch_t<256, 4, 1, false, true>(p, grid, block, smem, s, win)
+                              : launch_t<256, 4, 0, false, true>(p, grid, block, smem, s, win);
     if (p.n_req > 0) return p.any_fluence ? launch_m<3>(p, grid, block, threads_per_sm, smem, s, win)
                                            : launch_m<2>(p, grid, block, threads_per_sm, smem, s, win);
     return p.one.fl_n > 0 ? launch_m<1>(p, grid, block, threads_per_sm, smem, s, win)
