@@ -49,7 +49,8 @@ typedef struct {
     void *stream;             /* cudaStream_t to launch on; NULL: the context makes one */
     int blocks_per_sm;        /* transport grid = SMs x blocks_per_sm (default 4)     */
     int threads_per_block;    /* multiple of 32, <= 256 (default 256)                */
-    int chunk;                /* histories a warp claims at a time (default 256)      */
+    int chunk;                /* histories a warp claims at a time (default 256; at most 32
+                                 of a launch's last ones, some 128 per warp)          */
     int flight_cap;           /* Woodcock flights a lane takes in a row, stopping early at a
                                  real interaction, before its warp moves on (default 4) */
     int multi_blocks_per_sm;  /* grid of multi-request launches (batched, served; default 3) */
@@ -158,7 +159,7 @@ typedef struct {
     double d_max;            /* Gy per history                                            */
     double t_total_s;        /* wall time of the run call                                 */
     double t_transport_s;    /* device time of the transport kernels (CUDA events)        */
-    int transport_launches;
+    int transport_launches;  /* batches whose tallies fit side by side into 1 GiB share one */
 } ctd_run_stats;
 
 /* Thread-local message of the last failed call on this thread. */

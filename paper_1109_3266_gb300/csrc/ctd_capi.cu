@@ -235,6 +235,7 @@ void fill_request(Phantom &P, uint64_t seed, ctd::RequestDesc &q)
     q.mmax = P.mm.p;
     q.rsurf = P.rs.p;
     q.csurf = P.cs.p;
+    q.pref = P.pref.p;
     q.cs_stride = P.phys.compton_model == CTD_COMPTON_WH ? (P.n_e - 1) * (P.phys.n_zeta - 1) : 0;
     if (P.fl_nu > 0) {
         q.fl_thr = P.fl_thr.p;
@@ -390,9 +391,44 @@ int finish_stats(Phantom &P, int nb, cudaStream_t s)
     return e;
 }
 
-// One transport launch over local histories [lb, le) of a batch starting at global h_base.
-int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, int which_size, uint64_t h_base, uint64_t lb,
-              uint64_t le, double *tally, size_t ev_index, uint4 *trace, uint64_t trace_h0, uint64_t trace_n,
+// Claims: runs of `chunk` histories until what is left is some 128 per warp, then of
+// 32, one round of source photons.  A launch of fewer histories takes 32 (or, below 32
+// a warp, down to 8) from the start: with claims of 256 alone, 1.4e5 histories went to
+// 558 of 4864 warps.
+void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1, double *tally, uint32_t stride,
+               int chunk, int warps)
+{
+    q.n_lo = n / nb;
+    q.rem = n % nb;
+    const uint64_t larger = q.rem * (q.n_lo + 1);   // histories in the larger batches
+    q.b0 = static_cast<int>(h0 < larger ? h0 / (q.n_lo + 1) : q.rem + (h0 - larger) / q.n_lo);
+    q.h_begin = h0;
+    q.h_end = h1;
+    const uint64_t w = static_cast<uint64_t>(std::max(warps, 1)), tail = 128 * w, count = h1 - h0;
+    q.h_big = count > tail ? h1 - tail : h0;
+    q.small = static_cast<int>(std::min<uint64_t>(std::max<uint64_t>(count / w, 8), 32));
+    q.small = std::min(q.small, chunk);
+    q.tally = tally;
+    q.tally_stride = stride;
+}
+
+ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, double *tally, bool clear)
+{
+    // d = E / (m n_b) with m = rho V / 1000 kg
+    const double vol = P.dx * P.dy * P.dz;
+    const uint64_t n_lo = n / nb, rem = n % nb;
+    ctd::FoldBatches f;
+    f.tally = tally;
+    f.nb = k;
+    f.n_first = static_cast<int>(std::min<uint64_t>(static_cast<uint64_t>(k), rem > static_cast<uint64_t>(b0) ? rem - b0 : 0));
+    f.scale0 = ctd::kKevToJ * 1000.0 / (vol * static_cast<double>(n_lo + 1));
+    f.scale1 = ctd::kKevToJ * 1000.0 / (vol * static_cast<double>(n_lo));
+    f.clear = clear;
+    return f;
+}
+
+int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1,
+              double *tally, uint32_t stride, size_t ev_index, uint4 *trace, uint64_t trace_h0, uint64_t trace_n,
               cudaStream_t s, unsigned long long *work)
 {
     if (!s) s = ctx->stream;
@@ -403,11 +439,7 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, int which_size, uin
     L.trace_h0 = trace_h0;
     L.trace_n = trace_n;
     fill_shared(P, L.sh);
-    q.pref = P.pref.p + which_size * (q.nbins + 1);
-    q.h_base = h_base;
-    q.local_begin = lb;
-    q.local_end = le;
-    q.tally = tally;
+    set_range(q, n, nb, h0, h1, tally, stride, ctx->chunk, ctx->num_sms * ctx->blocks_per_sm * ctx->threads / 32);
     q.work = work;
     L.one = q;
     L.chunk = ctx->chunk;
@@ -962,7 +994,16 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
     const size_t nv = P->nvox;
     const bool two = ctx->plain_overlap;
     if (two && (rc = ensure_plain_aux(ctx, *P))) return rc;
-    CK(cudaMemsetAsync(P->tally.p, 0, nv * sizeof(double), ctx->stream));
+    // Batches that share a launch have a tally each, in scratch memory while the call
+    // runs; without room for it (or where launches are per batch) the phantom's one.
+    Scratch scratch(&ctx->buffers, ctx->stream);
+    int group = two || ctx->l2_persist ? 1 : tallies_within(nv, n_batches, kTallyBudget);
+    if (group > 1 && scratch.buf.ensure(nv * group)) {
+        g_error.clear();
+        group = 1;
+    }
+    double *const tallies = group > 1 ? scratch.buf.p : P->tally.p;
+    CK(cudaMemsetAsync(tallies, 0, nv * group * sizeof(double), ctx->stream));
     if (two) CK(cudaMemsetAsync(P->tally2.p, 0, nv * sizeof(double), ctx->stream));
     CK(cudaMemsetAsync(P->sum_d.p, 0, nv * sizeof(double), ctx->stream));
     CK(cudaMemsetAsync(P->sum_d2.p, 0, nv * sizeof(double), ctx->stream));
@@ -970,46 +1011,55 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
     CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
     ctd::RequestDesc T;
     fill_request(*P, seed, T);
-    const uint64_t n_lo = n_histories / n_batches, rem = n_histories % n_batches;
-    const double vol = P->dx * P->dy * P->dz;
-    if (two) {
-        CK(cudaEventRecord(ctx->plain_fork, ctx->stream));
-        CK(cudaStreamWaitEvent(ctx->plain_aux, ctx->plain_fork, 0));
+    size_t launches = 0;
+    if (!two && !ctx->l2_persist) {
+        // batches share a launch, each with a tally of its own (run_request: no waiting for
+        // a batch's last histories), and are folded in order afterwards
+        for (int b = 0; b < n_batches; b += group) {
+            const int k = std::min(group, n_batches - b);
+            if (b > 0) CK(cudaMemsetAsync(tallies, 0, nv * k * sizeof(double), ctx->stream));
+            if ((rc = transport(ctx, *P, T, n_histories, n_batches, batch_start(n_histories, n_batches, b),
+                                batch_start(n_histories, n_batches, b + k), tallies, static_cast<uint32_t>(nv), launches)))
+                return rc;
+            ++launches;
+            CKS(ctd::launch_fold(fold_of(*P, n_histories, n_batches, b, k, tallies, false), P->rinv.p, P->sum_d.p,
+                                 P->sum_d2.p, P->edep.p, nv, ctx->stream));
+        }
+    } else {
+        if (two) {
+            CK(cudaEventRecord(ctx->plain_fork, ctx->stream));
+            CK(cudaStreamWaitEvent(ctx->plain_aux, ctx->plain_fork, 0));
+        }
+        // With two streams, odd batches run on the second one with the second tally: a
+        // batch's launch waits only for the fold two batches back (same stream, same
+        // tally), so it starts while the previous batch drains; each fold waits for the
+        // previous batch's fold, so Sigma d and Sigma d^2 add up in batch order.
+        for (int b = 0; b < n_batches; ++b) {
+            const int k = two ? b & 1 : 0;
+            const cudaStream_t s = k ? ctx->plain_aux : ctx->stream;
+            double *tally = k ? P->tally2.p : P->tally.p;
+            if ((rc = transport(ctx, *P, T, n_histories, n_batches, batch_start(n_histories, n_batches, b),
+                                batch_start(n_histories, n_batches, b + 1), tally, 0, b, nullptr, 0, 0, s, P->work.p + k)))
+                return rc;
+            if (two && b > 0) CK(cudaStreamWaitEvent(s, ctx->plain_fold[k ^ 1], 0));
+            CKS(ctd::launch_fold(fold_of(*P, n_histories, n_batches, b, 1, tally, true), P->rinv.p, P->sum_d.p,
+                                 P->sum_d2.p, P->edep.p, nv, s));
+            if (two) CK(cudaEventRecord(ctx->plain_fold[k], s));
+        }
+        launches = n_batches;
+        // the context's stream continues after the last fold (which followed every other)
+        if (two && ((n_batches - 1) & 1)) CK(cudaStreamWaitEvent(ctx->stream, ctx->plain_fold[1], 0));
     }
-    // With two streams, odd batches run on the second one with the second tally: a
-    // batch's launch waits only for the fold two batches back (same stream, same
-    // tally), so it starts while the previous batch drains; each fold waits for the
-    // previous batch's fold, so Sigma d and Sigma d^2 add up in batch order.
-    uint64_t h = 0;
-    for (int b = 0; b < n_batches; ++b) {
-        const uint64_t nb = static_cast<uint64_t>(b) < rem ? n_lo + 1 : n_lo;
-        const int which = static_cast<uint64_t>(b) < rem ? 0 : 1;
-        const int k = two ? b & 1 : 0;
-        const cudaStream_t s = k ? ctx->plain_aux : ctx->stream;
-        double *tally = k ? P->tally2.p : P->tally.p;
-        if ((rc = transport(ctx, *P, T, which, h, 0, nb, tally, b, nullptr, 0, 0, s, P->work.p + k))) return rc;
-        if (two && b > 0) CK(cudaStreamWaitEvent(s, ctx->plain_fold[k ^ 1], 0));
-        // d = E / (m n_b) with m = rho V / 1000 kg
-        const double scale = ctd::kKevToJ * 1000.0 / (vol * static_cast<double>(nb));
-        CKS(ctd::launch_fold(tally, P->rinv.p, P->sum_d.p, P->sum_d2.p, P->edep.p, nv, scale, s));
-        if (two) CK(cudaEventRecord(ctx->plain_fold[k], s));
-        h += nb;
-    }
-    // the context's stream continues after the last fold (which followed every other)
-    if (two && ((n_batches - 1) & 1)) CK(cudaStreamWaitEvent(ctx->stream, ctx->plain_fold[1], 0));
     CKS(ctd::launch_finalize(P->sum_d.p, P->sum_d2.p, n_batches, P->dose.p, P->sd.p, nv, ctx->stream));
     CKS(ctd::launch_rsd(P->dose.p, P->sd.p, P->rho.p, nv, P->partials.p, kRsdParts, P->result.p, ctx->stream));
     CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p + 5 * kRsdParts, kRsdParts, P->result.p + 3, ctx->stream));
-    if ((rc = collect(ctx, *P, n_batches, t0))) return rc;
+    if ((rc = collect(ctx, *P, launches, t0))) return rc;
+    scratch.idle = true;
     P->stats.histories = n_histories;
     P->stats.n_batches = n_batches;
     P->have_result = true;
     return CTD_OK;
 }
-
-}  // extern "C"
-
-extern "C" {
 
 int ctd_run_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, int n_batches, uint64_t h_begin,
                   uint64_t h_end, int clear)
@@ -1032,18 +1082,11 @@ int ctd_run_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t s
     P->have_result = false;
     ctd::RequestDesc T;
     fill_request(*P, seed, T);
-    const uint64_t n_lo = n_histories / n_batches, rem = n_histories % n_batches;
-    uint64_t h = 0;
+    // every batch deposits into the one grid
     size_t launches = 0;
-    for (int b = 0; b < n_batches; ++b) {
-        const uint64_t nb = static_cast<uint64_t>(b) < rem ? n_lo + 1 : n_lo;
-        const uint64_t lo = h_begin > h ? h_begin : h, hi = h_end < h + nb ? h_end : h + nb;
-        if (lo < hi) {
-            if ((rc = transport(ctx, *P, T, static_cast<uint64_t>(b) < rem ? 0 : 1, h, lo - h, hi - h, P->edep.p, launches)))
-                return rc;
-            ++launches;
-        }
-        h += nb;
+    if (h_begin < h_end) {
+        if ((rc = transport(ctx, *P, T, n_histories, n_batches, h_begin, h_end, P->edep.p, 0, launches))) return rc;
+        ++launches;
     }
     CK(cudaMemsetAsync(P->result.p, 0, 3 * sizeof(double), ctx->stream));
     CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p + 5 * kRsdParts, kRsdParts, P->result.p + 3, ctx->stream));
@@ -1076,16 +1119,6 @@ int ctd_shard_begin(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t
     return CTD_OK;
 }
 
-// batch b of the sharded run: its size, which allocation it uses, its first history
-static void shard_batch_of(const Phantom &P, int b, uint64_t &size, int &which, uint64_t &h0)
-{
-    const uint64_t n_lo = P.shard_n / P.shard_nb, rem = P.shard_n % P.shard_nb;
-    const uint64_t ub = static_cast<uint64_t>(b);
-    size = ub < rem ? n_lo + 1 : n_lo;
-    which = ub < rem ? 0 : 1;
-    h0 = ub * n_lo + (ub < rem ? ub : rem);
-}
-
 int ctd_shard_batch(ctd_ctx *ctx, ctd_phantom ph, int batch, uint64_t local_begin, uint64_t local_end,
                     double *tally_dev)
 {
@@ -1096,16 +1129,16 @@ int ctd_shard_batch(ctd_ctx *ctx, ctd_phantom ph, int batch, uint64_t local_begi
     if (P->shard_nb == 0) return fail(CTD_EINVAL, "no sharded run begun on phantom %d", ph);
     if (batch < 0 || batch >= P->shard_nb) return fail(CTD_EINVAL, "batch %d outside [0, %d)", batch, P->shard_nb);
     if (!tally_dev) return fail(CTD_EINVAL, "null tally buffer");
-    uint64_t size, h0;
-    int which;
-    shard_batch_of(*P, batch, size, which, h0);
+    const uint64_t h0 = batch_start(P->shard_n, P->shard_nb, batch);
+    const uint64_t size = batch_start(P->shard_n, P->shard_nb, batch + 1) - h0;
     if (local_begin > local_end || local_end > size)
         return fail(CTD_EINVAL, "history range outside batch %d of %llu histories", batch,
                     static_cast<unsigned long long>(size));
     if (local_begin == local_end) return CTD_OK;
     ctd::RequestDesc T;
     fill_request(*P, P->shard_seed, T);
-    return transport(ctx, *P, T, which, h0, local_begin, local_end, tally_dev, static_cast<size_t>(batch));
+    return transport(ctx, *P, T, P->shard_n, P->shard_nb, h0 + local_begin, h0 + local_end, tally_dev, 0,
+                     static_cast<size_t>(batch));
 }
 
 int ctd_shard_fold(ctd_ctx *ctx, ctd_phantom ph, int batch, double *tally_dev)
@@ -1117,12 +1150,8 @@ int ctd_shard_fold(ctd_ctx *ctx, ctd_phantom ph, int batch, double *tally_dev)
     if (P->shard_nb == 0) return fail(CTD_EINVAL, "no sharded run begun on phantom %d", ph);
     if (batch < 0 || batch >= P->shard_nb) return fail(CTD_EINVAL, "batch %d outside [0, %d)", batch, P->shard_nb);
     if (!tally_dev) return fail(CTD_EINVAL, "null tally buffer");
-    uint64_t size, h0;
-    int which;
-    shard_batch_of(*P, batch, size, which, h0);
-    // d = E / (m n_b) with m = rho V / 1000 kg
-    const double scale = ctd::kKevToJ * 1000.0 / (P->dx * P->dy * P->dz * static_cast<double>(size));
-    CKS(ctd::launch_fold(tally_dev, P->rinv.p, P->sum_d.p, P->sum_d2.p, P->edep.p, P->nvox, scale, ctx->stream));
+    CKS(ctd::launch_fold(fold_of(*P, P->shard_n, P->shard_nb, batch, 1, tally_dev, true), P->rinv.p, P->sum_d.p,
+                         P->sum_d2.p, P->edep.p, P->nvox, ctx->stream));
     return CTD_OK;
 }
 
@@ -1197,19 +1226,11 @@ int ctd_trace_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t
     P->have_result = false;
     ctd::RequestDesc T;
     fill_request(*P, seed, T);
-    const uint64_t n_lo = n_histories / n_batches, rem = n_histories % n_batches;
-    uint64_t h = 0;
+    // every batch deposits into the one grid
     size_t launches = 0;
-    for (int b = 0; b < n_batches; ++b) {
-        const uint64_t nb = static_cast<uint64_t>(b) < rem ? n_lo + 1 : n_lo;
-        const uint64_t lo = h_begin > h ? h_begin : h, hi = h_end < h + nb ? h_end : h + nb;
-        if (lo < hi) {
-            if ((rc = transport(ctx, *P, T, static_cast<uint64_t>(b) < rem ? 0 : 1, h, lo - h, hi - h, P->edep.p,
-                                launches, rec.p, h_begin, n)))
-                return rc;
-            ++launches;
-        }
-        h += nb;
+    if (h_begin < h_end) {
+        if ((rc = transport(ctx, *P, T, n_histories, n_batches, h_begin, h_end, P->edep.p, 0, launches, rec.p, h_begin, n))) return rc;
+        ++launches;
     }
     CK(cudaMemsetAsync(P->result.p, 0, 3 * sizeof(double), ctx->stream));
     CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p + 5 * kRsdParts, kRsdParts, P->result.p + 3, ctx->stream));

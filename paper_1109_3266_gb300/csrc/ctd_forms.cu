@@ -45,6 +45,28 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     if ((rc = ctx->u_work.ensure(static_cast<size_t>(n_batches) * n_req))) return rc;
     // descriptors for every batch of every request, the history and tile offsets
     std::vector<ctd::RequestDesc> descs(static_cast<size_t>(n_batches) * n_req);
+    // Request chains: batches of a request share launches as in a plain run, each with a
+    // tally in the call's scratch memory (requests whose batches would not fit side by
+    // side, or all without room for the scratch, keep the phantom's one).
+    std::vector<int> step(n_req, 1);
+    std::vector<double *> tallies(n_req);
+    Scratch scratch(&ctx->buffers, ctx->stream);
+    if (!ctx->shared_launch) {
+        size_t total = 0;
+        for (int r = 0; r < n_req; ++r) {
+            step[r] = tallies_within(ps[r]->nvox, n_batches, kBatchTallyBudget / n_req);
+            if (step[r] > 1) total += ps[r]->nvox * step[r];
+        }
+        if (total && scratch.buf.ensure(total)) {
+            g_error.clear();
+            step.assign(n_req, 1);
+        }
+    }
+    size_t taken = 0;
+    for (int r = 0; r < n_req; ++r) {
+        tallies[r] = step[r] > 1 ? scratch.buf.p + taken : ps[r]->tally.p;
+        if (step[r] > 1) taken += ps[r]->nvox * step[r];
+    }
     std::vector<ctd::FoldDesc> folds(static_cast<size_t>(n_batches) * n_req);
     std::vector<uint64_t> tiles(n_req + 1, 0);
     for (int r = 0; r < n_req; ++r)
@@ -52,26 +74,24 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     for (int r = 0; r < n_req; ++r) {
         Phantom &P = *ps[r];
         const size_t nv = P.nvox;
-        CK(cudaMemsetAsync(P.tally.p, 0, nv * sizeof(double), ctx->stream));
+        if (ctx->shared_launch) CK(cudaMemsetAsync(P.tally.p, 0, nv * sizeof(double), ctx->stream));
         CK(cudaMemsetAsync(P.sum_d.p, 0, nv * sizeof(double), ctx->stream));
         CK(cudaMemsetAsync(P.sum_d2.p, 0, nv * sizeof(double), ctx->stream));
         CK(cudaMemsetAsync(P.edep.p, 0, nv * sizeof(double), ctx->stream));
         CK(cudaMemsetAsync(P.counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
         P.have_result = false;
-        const uint64_t n = n_histories[r], n_lo = n / n_batches, rem = n % n_batches;
+        const uint64_t n = n_histories[r];
         const double vol = P.dx * P.dy * P.dz;
-        uint64_t h = 0;
-        for (int b = 0; b < n_batches; ++b) {
-            const uint64_t nb = static_cast<uint64_t>(b) < rem ? n_lo + 1 : n_lo;
-            const int which = static_cast<uint64_t>(b) < rem ? 0 : 1;
+        for (int b = 0; b < n_batches; b += step[r]) {
+            // request chains: step[r] batches share a launch; shared launches: one batch
+            const int k = std::min(step[r], n_batches - b);
+            const uint64_t h0 = batch_start(n, n_batches, b), h1 = batch_start(n, n_batches, b + k);
             ctd::RequestDesc &q = descs[static_cast<size_t>(b) * n_req + r];
             fill_request(P, seeds[r], q);
+            set_range(q, n, n_batches, h0, h1, tallies[r], ctx->shared_launch ? 0 : static_cast<uint32_t>(nv), ctx->chunk,
+                      ctx->num_sms * ctx->threads / 32 *
+                          (ctx->shared_launch ? ctx->multi_blocks_per_sm : ctx->blocks_per_sm));
             q.work = ctx->u_work.p + static_cast<size_t>(b) * n_req + r;
-            q.pref = P.pref.p + which * (q.nbins + 1);
-            q.h_base = h;
-            q.local_begin = 0;
-            q.local_end = nb;
-            q.tally = P.tally.p;
             ctd::FoldDesc &f = folds[static_cast<size_t>(b) * n_req + r];
             f.tally = P.tally.p;
             f.rinv = P.rinv.p;
@@ -79,8 +99,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             f.sum_d2 = P.sum_d2.p;
             f.edep = P.edep.p;
             f.nvox = nv;
-            f.scale = ctd::kKevToJ * 1000.0 / (vol * static_cast<double>(nb));
-            h += nb;
+            f.scale = ctd::kKevToJ * 1000.0 / (vol * static_cast<double>(h1 - h0));
         }
     }
     std::vector<unsigned char> key;
@@ -114,6 +133,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
         std::stable_sort(order.begin(), order.end(),
                          [&](int a, int b) { return n_histories[a] > n_histories[b]; });
         put(order.data(), order.size() * sizeof(int));
+        put(step.data(), step.size() * sizeof(int));
         body = [&, order, n_lanes](cudaStream_t cs) {
             if (cudaMemsetAsync(ctx->u_work.p, 0, static_cast<size_t>(n_batches) * n_req * sizeof(unsigned long long),
                                 cs) != cudaSuccess ||
@@ -125,12 +145,14 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
                 Phantom &P = *ps[r];
                 // the k-th largest request on lane k (mod the lanes)
                 const cudaStream_t ls = ctx->lanes[k % n_lanes];
-                for (int b = 0; b < n_batches && e == CTD_OK; ++b) {
+                for (int b = 0; b < n_batches && e == CTD_OK; b += step[r]) {
                     const size_t d = static_cast<size_t>(b) * n_req + r;
-                    e = launch_one(ctx, P, descs[d], ls);
+                    const int g = std::min(step[r], n_batches - b);
+                    if (cudaMemsetAsync(tallies[r], 0, P.nvox * g * sizeof(double), ls) != cudaSuccess) e = CTD_ECUDA;
+                    if (e == CTD_OK) e = launch_one(ctx, P, descs[d], ls);
                     if (e == CTD_OK)
-                        e = ctd::launch_fold(P.tally.p, P.rinv.p, P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, folds[d].scale,
-                                             ls);
+                        e = ctd::launch_fold(fold_of(P, n_histories[r], n_batches, b, g, tallies[r], false), P.rinv.p,
+                                             P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, ls);
                 }
                 if (e == CTD_OK) e = finish_stats(P, n_batches, ls);
             }
@@ -227,6 +249,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     }
     CK(cudaGraphLaunch(ctx->batch_graph, ctx->stream));
     if ((rc = collect_many(ctx, ps.data(), n_req, n_launch, t0))) return rc;
+    scratch.idle = true;
     for (int r = 0; r < n_req; ++r) {
         ps[r]->stats.histories = n_histories[r];
         ps[r]->stats.n_batches = n_batches;
@@ -408,20 +431,22 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
     ctd::RequestDesc q;
     fill_request(P, R.req.seed, q);
     q.work = ctx->serve_work.p + R.lane;
-    q.pref = P.pref.p + 1 * (q.nbins + 1);    // batches of exactly B histories
-    q.tally = P.tally.p;
-    const double scale = ctd::kKevToJ * 1000.0 / (P.dx * P.dy * P.dz * static_cast<double>(B));
+    // batches of exactly B histories (of a problem that ends with these)
+    const int nb = R.batches + std::max(n, 1);
+    const int warps = ctx->num_sms * ctx->blocks_per_sm * ctx->threads / 32;
     double hist = 0.0;
     for (int j = 0; j < std::max(n, 1); ++j) {
-        q.h_base = static_cast<uint64_t>(R.batches + j) * B;
-        q.local_begin = j == 0 ? lo : 0;
-        q.local_end = j == 0 ? hi : B;
-        if (q.local_begin < q.local_end) {
+        const uint64_t first = static_cast<uint64_t>(R.batches + j) * B;
+        const uint64_t h0 = j == 0 ? first + lo : first, h1 = j == 0 ? first + hi : first + B;
+        if (h0 < h1) {
+            set_range(q, B * nb, nb, h0, h1, P.tally.p, 0, ctx->chunk, warps);
             CK(cudaMemsetAsync(q.work, 0, sizeof(unsigned long long), s));
             CKS(launch_one(ctx, P, q, s));
-            hist += static_cast<double>(q.local_end - q.local_begin);
+            hist += static_cast<double>(h1 - h0);
         }
-        if (j < n) CKS(ctd::launch_fold(P.tally.p, P.rinv.p, P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, scale, s));
+        if (j < n)
+            CKS(ctd::launch_fold(fold_of(P, B * nb, nb, R.batches + j, 1, P.tally.p, true), P.rinv.p, P.sum_d.p,
+                                 P.sum_d2.p, P.edep.p, P.nvox, s));
         if (j == n - 2) CK(cudaEventRecord(ctx->serve_ev_pre[R.lane], s));
     }
     const int done = R.batches + n;
@@ -635,11 +660,9 @@ int serve_round(ctd_ctx *ctx)
         ctd::RequestDesc &q = descs[i];
         fill_request(P, R.req.seed, q);
         q.work = ctx->u_work.p + i;
-        q.pref = P.pref.p + 1 * (q.nbins + 1);    // batches of exactly B histories
-        q.h_base = static_cast<uint64_t>(R.batches) * B;
-        q.local_begin = 0;
-        q.local_end = B;
-        q.tally = P.tally.p;
+        // batch R.batches of a problem of R.batches + 1 batches of exactly B histories
+        set_range(q, B * (R.batches + 1), R.batches + 1, B * R.batches, B * (R.batches + 1), P.tally.p, 0, ctx->chunk,
+                  ctx->num_sms * ctx->multi_blocks_per_sm * ctx->threads / 32);
         tiles[i + 1] = tiles[i] + (P.nvox + ctd::kFoldTile - 1) / ctd::kFoldTile;
         ctd::FoldDesc &f = folds[i];
         f.tally = P.tally.p;

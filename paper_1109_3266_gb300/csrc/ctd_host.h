@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <array>
 #include <cstdint>
 #include <map>
@@ -162,6 +163,19 @@ struct Phantom {
     }
 };
 
+// Device scratch of one call, taken from the context's released buffers and given back
+// when the call ends, then idle (after a failed call the stream is waited for first).
+struct Scratch {
+    DevBuf<double> buf;
+    cudaStream_t stream;
+    bool idle = false;
+    Scratch(BufferCache *c, cudaStream_t s) : stream(s) { buf.cache = c; }
+    ~Scratch()
+    {
+        if (buf.p && !idle) cudaStreamSynchronize(stream);
+    }
+};
+
 struct Staged {
     ctd::DeviceCounts c;
     double res[4];    // avg RSD, sigma_bar, D_max, deposited energy
@@ -189,6 +203,9 @@ struct ServeReq {
     bool in_flight = false, checked = false, split = false;
 };
 
+// device memory a plain run may take, while it runs, for the tallies of batches that
+// share a launch, and a batched call for all its requests'
+constexpr size_t kTallyBudget = size_t(1) << 30, kBatchTallyBudget = size_t(512) << 20;
 constexpr int kRsdParts = 1024;   // partial sums of the statistics reductions
 constexpr int kMaxLanes = 64;     // streams for request chains
 constexpr uint64_t kMaxTrace = 1ull << 26;   // histories of one trace call (16 B of device memory each)
@@ -296,12 +313,32 @@ int join_lanes(ctd_ctx *ctx, cudaStream_t origin, int n);
 int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t s);
 // mean, standard error, avg RSD and deposited energy of nb finished batches
 int finish_stats(Phantom &P, int nb, cudaStream_t s);
-// one transport launch over local histories [lb, le) of a batch starting at h_base,
-// bracketed by timing events 2 ev_index and 2 ev_index + 1
+// q covers histories [h0, h1) of the problem of n histories in nb batches, deposits of
+// its first batch into tally and of each later one `stride` voxels further on, for a
+// launch of `warps` warps
+void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1, double *tally, uint32_t stride,
+               int chunk, int warps);
+// batch b of n histories in nb batches: its first history
+inline uint64_t batch_start(uint64_t n, int nb, int b)
+{
+    const uint64_t n_lo = n / nb, rem = n % nb, ub = static_cast<uint64_t>(b);
+    return ub * n_lo + (ub < rem ? ub : rem);
+}
+// how many of nb batches' tallies of nvox voxels fit side by side into budget bytes
+// (one at least; voxel offsets are 32-bit on the device)
+inline int tallies_within(size_t nvox, int nb, size_t budget)
+{
+    const size_t most = std::min(budget / (nvox * sizeof(double)), (static_cast<size_t>(1) << 32) / nvox);
+    return static_cast<int>(std::min<size_t>(std::max<size_t>(most, 1), static_cast<size_t>(nb)));
+}
+// fold of batches [b0, b0 + k) of the problem of n histories in nb batches from tally[k][nvox]
+ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, double *tally, bool clear);
+// one transport launch over histories [h0, h1) of n in nb batches (set_range), bracketed
+// by timing events 2 ev_index and 2 ev_index + 1
 // (trace: per-history records of histories trace_h0 .. trace_h0 + trace_n - 1, or nullptr)
 // on stream s (null: the context's) with claim counter work (null: the phantom's first)
-int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, int which_size, uint64_t h_base, uint64_t lb,
-              uint64_t le, double *tally, size_t ev_index, uint4 *trace = nullptr, uint64_t trace_h0 = 0,
+int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1,
+              double *tally, uint32_t stride, size_t ev_index, uint4 *trace = nullptr, uint64_t trace_h0 = 0,
               uint64_t trace_n = 0, cudaStream_t s = nullptr, unsigned long long *work = nullptr);
 double now_s();
 int transport_time(ctd_ctx *ctx, size_t n_launch, double &t);

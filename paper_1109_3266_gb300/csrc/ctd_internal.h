@@ -96,7 +96,7 @@ struct alignas(16) RequestDesc {
     // holds S[j][i], S[j][i+1], S[j+1][i], S[j+1][i+1], the corners of one bilinear lookup
     const float *rsurf;          // [n_mat] surfaces of cells
     const float *csurf;          // [n_c] surfaces of cells, material m at m * cs_stride cells
-    const uint64_t *pref;        // [nbins+1] bin starts inside the batch
+    const uint64_t *pref;        // [2][nbins+1] bin starts inside a batch of n_lo + 1 and of n_lo histories
     const float *bin_lo;         // [nbins]
     const float *bin_hi;         // [nbins]
     const float *cb;             // [n_proj]
@@ -104,10 +104,18 @@ struct alignas(16) RequestDesc {
     const float *zb;             // [n_proj] source height of each projection (helical)
     double *tally;               // [nvox] keV
     DeviceCounts *counts;
-    unsigned long long *work;    // claim counter over [local_begin, local_end)
+    unsigned long long *work;    // claim counter: histories claimed of [h_begin, h_end)
     uint64_t seed;
-    uint64_t h_base;             // global index of local index 0 (first history of the batch)
-    uint64_t local_begin, local_end;
+    // The launch runs histories [h_begin, h_end) of a problem whose batches are runs of
+    // consecutive histories, the first `rem` of n_lo + 1 and the others of n_lo: batch b
+    // starts at b n_lo + min(b, rem).  Deposits of batch b go to tally + (b - b0) tally_stride.
+    uint64_t h_begin, h_end;
+    uint64_t h_big;              // claims starting before it take P.chunk histories, later ones `small`
+    uint64_t n_lo, rem;
+    int b0;                      // batch of h_begin
+    uint32_t tally_stride;       // voxels, or 0: every batch into one grid
+    int small;
+    int pad_;
     int n_mat;
     int nbins;
     int nx, ny, nz;
@@ -203,12 +211,22 @@ struct L2Window {
     float hit_ratio;
 };
 
+// Batches of a fold: tallies tally[k][nvox], k < nb, the first n_first of a batch size
+// with scale0 = keV->J * 1000 / (V n_b) and the others with scale1.
+// With `clear` the tallies are left zeroed.
+struct FoldBatches {
+    double *tally;
+    int nb, n_first;
+    double scale0, scale1;
+    int clear;
+};
+
 // launches (ctd_transport.cu / ctd_stats.cu); win may be null
 int launch_transport(const LaunchParams &p, int grid, int block, int threads_per_sm, void *stream,
                      const L2Window *win = nullptr);
 size_t transport_smem_bytes(const LaunchParams &p, int threads);
-int launch_fold(double *tally, const double *rinv, double *sum_d, double *sum_d2, double *edep, size_t nvox,
-                double scale, void *stream);
+int launch_fold(const FoldBatches &f, const double *rinv, double *sum_d, double *sum_d2, double *edep, size_t nvox,
+                void *stream);
 int launch_finalize(const double *sum_d, const double *sum_d2, int nb, double *dose, double *sd, size_t nvox,
                     void *stream);
 int launch_rsd(const double *dose, const double *sd, const float *rho, size_t nvox, double *partials,

@@ -29,12 +29,8 @@ __device__ __forceinline__ double recip(double x)
     return fma(y, e, y);
 }
 
-// Fold one batch: d = E_b / (m_v n_b) in Gy per history; accumulate d and d^2,
-// keep the raw energy, clear the batch tally.  scale = keV->J * 1000 / (V n_b),
-// rinv = 1 / rho (0 where rho = 0).  Four voxels a grid stride apart per thread
-// and pass, so that their loads are in flight together.
-constexpr int kFoldUnroll = 4;
-
+// Fold batches in order: d = E_b / (m_v n_b) in Gy per history; accumulate d and d^2,
+// keep the raw energy, clear the tallies if asked.  rinv = 1 / rho (0 where rho = 0).
 __device__ __forceinline__ void fold_voxel(double t, size_t v, double *__restrict__ tally,
                                            const double *__restrict__ rinv, double *__restrict__ sum_d,
                                            double *__restrict__ sum_d2, double *__restrict__ edep, double scale)
@@ -46,21 +42,35 @@ __device__ __forceinline__ void fold_voxel(double t, size_t v, double *__restric
     sum_d2[v] += d * d;
 }
 
-__global__ void fold_kernel(double *__restrict__ tally, const double *__restrict__ rinv, double *__restrict__ sum_d,
-                            double *__restrict__ sum_d2, double *__restrict__ edep, size_t nvox, double scale)
+// One voxel per thread and pass, the sums in registers over its batches; the tallies
+// of kFoldUnroll batches are in flight together.  Bound by memory: per voxel 8 bytes a
+// batch and 56 once, where a fold per batch moved 64 bytes a batch.
+constexpr int kFoldUnroll = 4;
+
+__global__ void fold_kernel(const FoldBatches f, const double *__restrict__ rinv, double *__restrict__ sum_d,
+                            double *__restrict__ sum_d2, double *__restrict__ edep, size_t nvox)
 {
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
-    for (size_t v0 = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; v0 < nvox;
-         v0 += kFoldUnroll * stride) {
-        double t[kFoldUnroll];
+    for (size_t v = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; v < nvox; v += stride) {
+        const double r = rinv[v];
+        double s1 = sum_d[v], s2 = sum_d2[v], e = edep[v];
+        for (int b = 0; b < f.nb; b += kFoldUnroll) {
+            double t[kFoldUnroll];
 #pragma unroll
-        for (int k = 0; k < kFoldUnroll; ++k) {
-            const size_t v = v0 + k * stride;
-            t[k] = v < nvox ? tally[v] : 0.0;
+            for (int k = 0; k < kFoldUnroll; ++k) t[k] = b + k < f.nb ? f.tally[(b + k) * nvox + v] : 0.0;
+#pragma unroll
+            for (int k = 0; k < kFoldUnroll; ++k)
+                if (t[k] != 0.0) {
+                    const double d = (t[k] * (b + k < f.n_first ? f.scale0 : f.scale1)) * r;
+                    e += t[k];
+                    s1 += d;
+                    s2 += d * d;
+                    if (f.clear) f.tally[(b + k) * nvox + v] = 0.0;
+                }
         }
-#pragma unroll
-        for (int k = 0; k < kFoldUnroll; ++k)
-            if (t[k] != 0.0) fold_voxel(t[k], v0 + k * stride, tally, rinv, sum_d, sum_d2, edep, scale);
+        sum_d[v] = s1;
+        sum_d2[v] = s2;
+        edep[v] = e;
     }
 }
 
@@ -294,12 +304,10 @@ inline int ok() { return cudaGetLastError() == cudaSuccess ? CTD_OK : CTD_ECUDA;
 
 }  // namespace
 
-int launch_fold(double *tally, const double *rinv, double *sum_d, double *sum_d2, double *edep, size_t nvox,
-                double scale, void *stream)
+int launch_fold(const FoldBatches &f, const double *rinv, double *sum_d, double *sum_d2, double *edep, size_t nvox,
+                void *stream)
 {
-    const size_t per_pass = (nvox + kFoldUnroll - 1) / kFoldUnroll;
-    fold_kernel<<<grid_for(per_pass), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(tally, rinv, sum_d, sum_d2,
-                                                                                          edep, nvox, scale);
+    fold_kernel<<<grid_for(nvox), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(f, rinv, sum_d, sum_d2, edep, nvox);
     return ok();
 }
 

@@ -28,6 +28,7 @@ struct Photon {
     float x, y, z;    // position in voxel units: (r - box origin) / voxel size per axis
     float ux, uy, uz, e;
     uint64_t h;
+    uint32_t tally;   // first voxel of its batch's tally
     uint32_t step;
     int j;            // energy node of e, its fraction and 1 / the majorant there;
     float te, imax;   // they change only with e
@@ -158,26 +159,26 @@ __device__ __forceinline__ void flush_warp(DeviceCounts *dst, LaneCounts &c, uin
     __syncwarp();
 }
 
-__device__ __forceinline__ int bin_search(const RequestDesc &q, uint64_t local)
+__device__ __forceinline__ int bin_search(const uint64_t *pref, int nbins, uint64_t local)
 {
     // largest bin j with pref[j] <= local
-    int lo = 0, hi = q.nbins - 1;
+    int lo = 0, hi = nbins - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(&q.pref[mid]) <= local) lo = mid;
+        if (__ldg(&pref[mid]) <= local) lo = mid;
         else hi = mid - 1;
     }
     return lo;
 }
 
-// Source photon of local history `local` (global index h) of request q;
-// `bin` is a lower bound of its 1 keV interval.  Returns true if the photon
+// Source photon of history h of request q, history `local` of its batch, whose bin
+// starts are `pref`; `bin` is a lower bound of its 1 keV interval.  Returns true if the photon
 // enters the phantom.
 template <bool kKeys, bool kFluence, bool kTrace>
-__device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, uint64_t local, int bin, Photon &ph,
-                                       LaneCounts &cnt, const Tracer &tr)
+__device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, const uint64_t *pref, uint64_t local, int bin,
+                                       Photon &ph, LaneCounts &cnt, const Tracer &tr)
 {
-    while (bin < q.nbins - 1 && __ldg(&q.pref[bin + 1]) <= local) ++bin;
+    while (bin < q.nbins - 1 && __ldg(&pref[bin + 1]) <= local) ++bin;
     const U4 b0 = draw<kKeys>(q, h, 0, kStreamSource);
     const float elo = __ldg(&q.bin_lo[bin]), ehi = __ldg(&q.bin_hi[bin]);
     const float e = __fmaf_rn(ehi - elo, uni(b0.x), elo);
@@ -390,7 +391,7 @@ __device__ __forceinline__ int interact(const SharedTables &sh, const RequestDes
     const bool absorbed = pe || cutoff;
     ph.e = compton && !cutoff ? ec : e;
     const float dep = absorbed ? e : e - ph.e;
-    deposit(q.tally, at.idx, dep);
+    deposit(q.tally, at.idx + ph.tally, dep);
     cnt.compton += compton;
     cnt.rayleigh += rayleigh;
     int end = pe ? kDonePe : cutoff ? kDoneCutoff : kNotEnded;
@@ -413,34 +414,72 @@ __device__ __forceinline__ int interact(const SharedTables &sh, const RequestDes
 // Per-warp photon queue in shared memory: source photons are made 32 at a
 // time by the whole warp and taken by lanes whose history has ended.
 constexpr int kQueue = 48, kQueueLow = 16;
-constexpr size_t kQueueBytes = kQueue * (2 * sizeof(float4) + sizeof(uint64_t));
+constexpr size_t kQueueBytes = 3 * kQueue * sizeof(float4);
 
-// A warp's claim of local history indices [next, end), the 1 keV interval of its
-// first history and the source photons the warp has made, kept in shared memory
-// (read only when the queue is topped up).
+// A warp's claim of histories [next, end) and what holds up to `lim`, the end of
+// the claim or of the batch of `next`: the batch, its first history, its bin starts,
+// the 1 keV interval of a history at or before `next` and the first voxel of its
+// tally.  Kept in shared memory, read only when the queue is topped up.
 struct WarpPool {
-    uint64_t next, end, sourced;
-    int bin;
+    uint64_t next, lim, end, first, sourced;   // sourced: histories the warp has claimed
+    const uint64_t *pref;
+    int batch, bin;
+    uint32_t tally;
     int pad;
 };
 
 // Photons in vectors, so that one is stored or taken with three wide accesses; the
 // inverse majorant is worked out by the whole warp that made the photon.  Topped up
-// below 16 photons: 47 at most, and the tables, queues and slots of 32 warps leave
+// below 16 photons: 47 at most, and the tables, queues and slots of an SM's warps leave
 // L1 more than 60 KB (with 28 KB, the largest shared-memory carve-out, CBCT water
 // took 9 % longer: the gathers' lines in flight need it).
 struct Queue {
     float4 *a;     // [kQueue] x, y, z (voxel units), ux
-    float4 *b;     // [kQueue] uy, uz, e, 1 / mu_max(e)
-    uint64_t *h;   // [kQueue]
+    float4 *b;     // [kQueue] uy, uz, e, te
+    uint4 *c;      // [kQueue] h (lo, hi), first voxel of the batch's tally, bits of 1 / mu_max(e)
     WarpPool *pool;
+    __device__ __forceinline__ void put(int slot, const Photon &ph) const
+    {
+        a[slot] = make_float4(ph.x, ph.y, ph.z, ph.ux);
+        b[slot] = make_float4(ph.uy, ph.uz, ph.e, ph.te);
+        c[slot] = make_uint4(static_cast<uint32_t>(ph.h), static_cast<uint32_t>(ph.h >> 32), ph.tally,
+                             __float_as_uint(ph.imax));
+    }
+    // all but the step; the node follows from e and te
+    __device__ __forceinline__ void get(int slot, Photon &ph, int e_min) const
+    {
+        const float4 u = a[slot], v = b[slot];
+        const uint4 w = c[slot];
+        ph.x = u.x;
+        ph.y = u.y;
+        ph.z = u.z;
+        ph.ux = u.w;
+        ph.uy = v.x;
+        ph.uz = v.y;
+        ph.e = v.z;
+        ph.te = v.w;
+        ph.h = w.x | (static_cast<uint64_t>(w.y) << 32);
+        ph.tally = w.z;
+        ph.imax = __uint_as_float(w.w);
+        // te = (e - e_min) - j exactly, so j is exact and this its bit pattern
+        ph.j = static_cast<int>(__float_as_uint(((ph.e - static_cast<float>(e_min)) - ph.te) + kTrunc) - kTruncBits);
+    }
 };
 
 constexpr size_t kWarpBytes = kQueueBytes + sizeof(WarpPool) + 32 * sizeof(LaneSlot);
 static_assert(kWarpBytes % 16 == 0, "a warp's shared-memory area must keep 16-byte alignment");
 
-// All histories [q.local_begin, q.local_end) of one request, claimed by warps
-// from q.work in runs of `chunk`.  Returns when the warp has no photon left.
+// All histories [q.h_begin, q.h_end) of one request, claimed by warps from q.work in
+// runs of P.chunk, near the end of q.small.  A claim's photons carry their batch's
+// tally with them, so a warp goes from one batch to the next without draining.
+// Returns when the warp has no photon left.
+//
+// One launch per batch waited for each batch's last histories: some fifty to a
+// hundred microseconds of a few deep histories and of warps with a claim of 256
+// beside warps with none, which is nearly all of a small batch.  Transport of 1e5
+// histories in 10 batches (32^3 water): 0.69 ms in 10 launches -> 0.071 in one; 1e6 in 7
+// (51x51x32 head) 2.83 -> 0.43; 1e7 in 10 (48x48x40 head, helix) 4.31 -> 1.47; 2e8 in 2
+// (CBCT water) 15.29 -> 15.00.
 template <bool kKeys, bool kFluence, bool kWide, bool kAnyMode, bool kTrace>
 __device__ __forceinline__ void run_request(const LaunchParams &P, const RequestDesc &q, const float2 *s_tab,
                                             const float *s_mm, const Queue &Q, int lane, LaneCounts &cnt)
@@ -450,61 +489,83 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
     tr.h0 = P.trace_h0;
     tr.n = kTrace ? P.trace_n : 0;
     const unsigned lt_mask = (1u << lane) - 1u;
-    Photon ph;
+    Photon ph{};
+    ph.e = static_cast<float>(P.sh.e_min);
     bool alive = false;
     bool drained = false;
     int qcount = 0;                         // photons waiting in the warp's queue
     if (lane == 0) {
-        Q.pool->next = 0;
-        Q.pool->end = 0;
-        Q.pool->sourced = 0;
-        Q.pool->bin = 0;
+        WarpPool w{};
+        w.next = w.lim = w.end = q.h_begin;
+        w.batch = q.b0;
+        w.first = static_cast<uint64_t>(q.b0) * q.n_lo + (static_cast<uint64_t>(q.b0) < q.rem ? q.b0 : q.rem);
+        *Q.pool = w;
     }
     __syncwarp();
     for (;;) {
         // top the queue up with one round of up to 32 source photons
         if (qcount < kQueueLow && !drained) {
-            uint64_t pool_next = Q.pool->next, pool_end = Q.pool->end;
-            int pool_bin = Q.pool->bin;
-            if (pool_next >= pool_end) {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(q.work, static_cast<unsigned long long>(P.chunk));
-                base = __shfl_sync(kFull, base, 0);
-                const uint64_t b = q.local_begin + base;
-                if (b >= q.local_end) {
-                    drained = true;
-                } else {
-                    pool_next = b;
-                    pool_end = b + P.chunk < q.local_end ? b + P.chunk : q.local_end;
-                    pool_bin = bin_search(q, pool_next);
+            uint64_t next = Q.pool->next;
+            if (next >= Q.pool->lim) {
+                // the claim is used up, or goes on in the next batch
+                uint64_t end = Q.pool->end, first = Q.pool->first;
+                int batch = Q.pool->batch;
+                if (next >= end) {
+                    const unsigned size = end < q.h_big ? P.chunk : q.small;
+                    unsigned long long base = 0;
+                    if (lane == 0) base = atomicAdd(q.work, static_cast<unsigned long long>(size));
+                    base = __shfl_sync(kFull, base, 0);
+                    next = q.h_begin + base;
+                    end = next + size < q.h_end ? next + size : q.h_end;
+                    drained = next >= q.h_end;
+                }
+                if (!drained) {
+                    uint64_t size = q.n_lo + (static_cast<uint64_t>(batch) < q.rem ? 1 : 0);
+                    while (next - first >= size) {
+                        first += size;
+                        ++batch;
+                        size = q.n_lo + (static_cast<uint64_t>(batch) < q.rem ? 1 : 0);
+                    }
+                    const uint64_t *pref = size > q.n_lo ? q.pref : q.pref + (q.nbins + 1);
+                    const int bin = bin_search(pref, q.nbins, next - first);
+                    __syncwarp();
+                    if (lane == 0) {
+                        Q.pool->sourced += next == Q.pool->next && Q.pool->end == end ? 0 : end - next;
+                        Q.pool->next = next;
+                        Q.pool->end = end;
+                        Q.pool->lim = end < first + size ? end : first + size;
+                        Q.pool->first = first;
+                        Q.pool->pref = pref;
+                        Q.pool->batch = batch;
+                        Q.pool->bin = bin;
+                        Q.pool->tally = static_cast<uint32_t>(batch - q.b0) * q.tally_stride;
+                    }
+                    __syncwarp();
                 }
             }
             if (!drained) {
-                const uint64_t avail = pool_end - pool_next;
+                const uint64_t avail = Q.pool->lim - next;
                 const unsigned take = avail < 32 ? static_cast<unsigned>(avail) : 32u;
+                // the lanes' own photons wait in the queue's free slots meanwhile, so that
+                // source sampling has the registers to itself
+                const int mine = qcount + lane;
+                Q.put(mine, ph);
+                __syncwarp();
                 Photon np;
                 bool ok = false;
-                if (lane < take) {
-                    const uint64_t local = pool_next + lane;
-                    ok = source<kKeys, kFluence, kTrace>(q, q.h_base + local, local, pool_bin, np, cnt, tr);
-                }
+                if (lane < take)
+                    ok = source<kKeys, kFluence, kTrace>(q, next + lane, Q.pool->pref, next - Q.pool->first + lane,
+                                                         Q.pool->bin, np, cnt, tr);
                 const unsigned okm = __ballot_sync(kFull, ok);
+                Q.get(mine, ph, P.sh.e_min);
+                __syncwarp();
                 if (ok) {
-                    const int slot = qcount + __popc(okm & lt_mask);
                     set_energy(np, P.sh, s_mm);
-                    Q.a[slot] = make_float4(np.x, np.y, np.z, np.ux);
-                    Q.b[slot] = make_float4(np.uy, np.uz, np.e, np.imax);
-                    Q.h[slot] = np.h;
+                    np.tally = Q.pool->tally;
+                    Q.put(qcount + __popc(okm & lt_mask), np);
                 }
                 qcount += __popc(okm);
-                pool_next += take;
-                if (lane == 0) Q.pool->sourced += take;
-            }
-            __syncwarp();
-            if (lane == 0) {
-                Q.pool->next = pool_next;
-                Q.pool->end = pool_end;
-                Q.pool->bin = pool_bin;
+                if (lane == 0) Q.pool->next = next + take;
             }
             __syncwarp();
         }
@@ -515,17 +576,7 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
             const int rank = __popc(need & lt_mask);
             if (rank < npop) {
                 const int slot = qcount - 1 - rank;
-                const float4 a = Q.a[slot], b = Q.b[slot];
-                ph.x = a.x;
-                ph.y = a.y;
-                ph.z = a.z;
-                ph.ux = a.w;
-                ph.uy = b.x;
-                ph.uz = b.y;
-                ph.e = b.z;
-                ph.imax = b.w;
-                ph.h = Q.h[slot];
-                ph.j = enode(ph.e, P.sh.e_min, P.sh.n_e, ph.te);
+                Q.get(slot, ph, P.sh.e_min);
                 ph.step = 0;
                 if (kAnyMode) cnt.me->nreal = 0;
                 alive = true;
@@ -610,7 +661,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
     Queue Q;
     Q.a = reinterpret_cast<float4 *>(wbase);
     Q.b = Q.a + kQueue;
-    Q.h = reinterpret_cast<uint64_t *>(Q.b + kQueue);
+    Q.c = reinterpret_cast<uint4 *>(Q.b + kQueue);
     Q.pool = reinterpret_cast<WarpPool *>(wbase + kQueueBytes);
     LaneCounts cnt;
     cnt.me = reinterpret_cast<LaneSlot *>(wbase + kQueueBytes + sizeof(WarpPool)) + lane;
@@ -635,7 +686,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
             for (int rr = r; rr < P.n_req; ++rr) {
                 const RequestDesc &c = P.reqs[rr];
                 const unsigned long long claimed = *reinterpret_cast<volatile unsigned long long *>(c.work);
-                if (c.local_begin + claimed < c.local_end) {
+                if (c.h_begin + claimed < c.h_end) {
                     found = rr;
                     break;
                 }

@@ -92,7 +92,7 @@ int ctd_autotune(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_probe, uint64_t seed, 
         for (int rep = 0; rep < 2; ++rep) {
             CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
             int e;
-            if ((e = transport(ctx, *P, q, 0, 0, 0, n, P->tally.p, 0))) return e;
+            if ((e = transport(ctx, *P, q, P->alloc_n, P->alloc_nb, 0, n, P->tally.p, 0, 0))) return e;
             CK(cudaStreamSynchronize(ctx->stream));
             float ms = 0.0f;
             CK(cudaEventElapsedTime(&ms, ctx->events[0], ctx->events[1]));

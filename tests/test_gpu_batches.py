@@ -1,0 +1,63 @@
+"""Batches that share a transport launch (each with its own tally, folded in order)
+against one launch per batch (the overlapped plain run), where the claims and the
+batch boundaries meet: batches of one history, of just under and over a warp's
+round, uneven batches, a launch with fewer histories than warps and one with more
+than the small claims at its end cover.  Same histories, so the counts are equal;
+deposits are binary32 numbers added in binary64, so the tallies differ by rounding
+of at most n 2^-53 relative, far below 1e-12 here."""
+import numpy as np
+import pytest
+
+from paper_1109_3266_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+COUNTS = ("pe", "compton", "rayleigh", "fictitious", "escaped", "missed", "cutoff", "terminated", "aborted", "steps")
+
+
+@pytest.fixture(scope="module")
+def ctd():
+    from paper_1109_3266_gb300 import build, ctd as binding
+    build.build()
+    return binding
+
+
+@pytest.fixture(scope="module")
+def contexts(ctd):
+    cs = [ctd.ctd_create(device=0), ctd.ctd_create(device=0, plain_overlap=1)]
+    yield cs
+    for c in cs:
+        ctd.ctd_destroy(c)
+
+
+@pytest.mark.parametrize("n,nb", [(2, 2), (50, 50), (1_000, 37), (31 * 9 + 4, 9), (100_003, 7), (3_000_001, 5)])
+def test_shared_launch_equals_launch_per_batch(ctd, contexts, n, nb):
+    p = I.head(n, nb, seed=11, shape=(40, 37, 25), d=0.6)
+    out = []
+    for c in contexts:
+        dose, sd, st, h = ctd.run_problem(c, p)
+        edep = ctd.ctd_get_edep(c, h, p.phantom.nvox)
+        ctd.ctd_destroy_phantom(c, h)
+        out.append((dose, sd, edep, st))
+    (d0, s0, e0, t0), (d1, s1, e1, t1) = out
+    assert t0["transport_launches"] == 1 and t1["transport_launches"] == nb
+    assert [t0[k] for k in COUNTS] == [t1[k] for k in COUNTS]
+    assert sum(t0[k] for k in ("pe", "cutoff", "escaped", "missed", "terminated", "aborted")) == n
+    assert t0["e_emitted_kev"] == t1["e_emitted_kev"] and t0["e_escaped_kev"] == t1["e_escaped_kev"]
+    assert np.allclose(e0, e1, rtol=1e-12, atol=0) and np.allclose(d0, d1, rtol=1e-12, atol=0)
+    # a variance is a difference of sums: its rounding is relative to the squared mean
+    assert np.allclose(s0 ** 2, s1 ** 2, rtol=1e-9, atol=1e-12 * float((d0 ** 2).max()))
+
+
+def test_batched_chains_share_launches_like_plain_runs(ctd, contexts):
+    ps = [I.head(10_007, 6, seed=3, shape=(24, 20, 16), d=1.0), I.cbct_water(200_001, 6, seed=4, shape=(32, 30, 8), d=0.8)]
+    c = contexts[0]
+    hs = [ctd.load_problem(c, p) for p in ps]
+    for _ in range(2):   # recorded, then replayed
+        ctd.ctd_run_batch(c, hs, [p.n_hist for p in ps], [p.seed for p in ps], 6)
+        got = [ctd.ctd_get_dose_and_stddev(c, h, p.phantom.nvox) for h, p in zip(hs, ps)]
+    for h, p, (dose, sd, st) in zip(hs, ps, got):
+        d1, s1, t1, _ = ctd.run_problem(contexts[1], p)
+        assert [st[k] for k in COUNTS] == [t1[k] for k in COUNTS]
+        assert np.allclose(dose, d1, rtol=1e-12, atol=0)
+        ctd.ctd_destroy_phantom(c, h)
