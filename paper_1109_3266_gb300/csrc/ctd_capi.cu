@@ -376,8 +376,8 @@ int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t
     L.one = q;
     L.chunk = ctx->chunk;
     L.flight_cap = ctx->flight_cap;
-    return ctd::launch_transport(L, ctx->num_sms * ctx->blocks_per_sm, ctx->threads,
-                                 ctx->threads * ctx->blocks_per_sm, s);
+    const LaunchShape shape = launch_shape(ctx, L.sh, q.mode, false);
+    return ctd::launch_transport(L, shape.grid, shape.block, shape.threads_per_sm, s);
 }
 
 // Mean, standard error, avg RSD and deposited energy of a finished run of nb
@@ -391,10 +391,29 @@ int finish_stats(Phantom &P, int nb, cudaStream_t s)
     return e;
 }
 
-// Claims: runs of `chunk` histories until what is left is some 128 per warp, then of
-// 32, one round of source photons.  A launch of fewer histories takes 32 (or, below 32
-// a warp, down to 8) from the start: with claims of 256 alone, 1.4e5 histories went to
-// 558 of 4864 warps.
+// The launch shape of a single request.  The default residency of 4 blocks of 256
+// threads per SM becomes 3 of 384 in full transport: 36 warps instead of 32 at 56
+// registers (54 used, no spills; blocks of a multiple of 128 threads load the four
+// schedulers alike).  Per 2e8 histories CBCT water 15.00 -> 14.93 ms, head 24.70 ->
+// 24.25, per 1e8 a 4 mm head 17.77 -> 17.45 (40 warps spill: 24.84).  Runs that limit
+// the real interactions are source-bound and stay (4.70 against 4.84 ms), as do shapes
+// the context's options ask for and the forms compiled for 256 threads only.
+LaunchShape launch_shape(const ctd_ctx *ctx, const ctd::SharedTables &sh, int mode, bool trace)
+{
+    ctd::LaunchParams L;
+    L.sh = sh;
+    L.n_req = 0;
+    // tables so large that three such blocks do not fit an SM's 228 KB (1 KB a block is reserved)
+    const bool fits = 3 * (ctd::transport_smem_bytes(L, 384) + 1024) <= 228 * 1024;
+    if (ctx->threads == 256 && ctx->blocks_per_sm == 4 && mode == CTD_MODE_FULL && !trace && !sh.wide && fits)
+        return {ctx->num_sms * 3, 384, 3 * 384};
+    return {ctx->num_sms * ctx->blocks_per_sm, ctx->threads, ctx->threads * ctx->blocks_per_sm};
+}
+
+// Claims: runs of `chunk` histories until what is left is some 256 per warp, then of
+// 32, one round of source photons.  1e6 histories (a 51x51x32 head, 183 per warp) took
+// 0.43 ms while half of them went in claims of 256, 0.24 in claims of 32; for 1e5 claims
+// of 18, so that every warp has one, took 0.080 ms, claims of 32 0.057.
 void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1, double *tally, uint32_t stride,
                int chunk, int warps)
 {
@@ -404,10 +423,9 @@ void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1
     q.b0 = static_cast<int>(h0 < larger ? h0 / (q.n_lo + 1) : q.rem + (h0 - larger) / q.n_lo);
     q.h_begin = h0;
     q.h_end = h1;
-    const uint64_t w = static_cast<uint64_t>(std::max(warps, 1)), tail = 128 * w, count = h1 - h0;
+    const uint64_t w = static_cast<uint64_t>(std::max(warps, 1)), tail = 256 * w, count = h1 - h0;
     q.h_big = count > tail ? h1 - tail : h0;
-    q.small = static_cast<int>(std::min<uint64_t>(std::max<uint64_t>(count / w, 8), 32));
-    q.small = std::min(q.small, chunk);
+    q.small = std::min(32, chunk);
     q.tally = tally;
     q.tally_stride = stride;
 }
@@ -439,7 +457,8 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb,
     L.trace_h0 = trace_h0;
     L.trace_n = trace_n;
     fill_shared(P, L.sh);
-    set_range(q, n, nb, h0, h1, tally, stride, ctx->chunk, ctx->num_sms * ctx->blocks_per_sm * ctx->threads / 32);
+    const LaunchShape shape = launch_shape(ctx, L.sh, q.mode, trace != nullptr);
+    set_range(q, n, nb, h0, h1, tally, stride, ctx->chunk, shape.grid * (shape.block / 32));
     q.work = work;
     L.one = q;
     L.chunk = ctx->chunk;
@@ -448,7 +467,6 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb,
     cudaEvent_t e0 = event_at(ctx, 2 * ev_index), e1 = event_at(ctx, 2 * ev_index + 1);
     if (!e0 || !e1) return fail(CTD_ECUDA, "cudaEventCreate failed");
     CK(cudaEventRecord(e0, s));
-    const int grid = ctx->num_sms * ctx->blocks_per_sm;
     ctd::L2Window win{};
     if (ctx->l2_persist) {
         // the tally's (or the voxel words') lines stay in L2
@@ -463,8 +481,7 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb,
         }
         win.hit_ratio = static_cast<float>(std::min(1.0, static_cast<double>(ctx->l2_setaside) / win.bytes));
     }
-    CKS(ctd::launch_transport(L, grid, ctx->threads, ctx->threads * ctx->blocks_per_sm, s,
-                              ctx->l2_persist ? &win : nullptr));
+    CKS(ctd::launch_transport(L, shape.grid, shape.block, shape.threads_per_sm, s, ctx->l2_persist ? &win : nullptr));
     CK(cudaEventRecord(e1, s));
     return CTD_OK;
 }

@@ -88,9 +88,12 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             const uint64_t h0 = batch_start(n, n_batches, b), h1 = batch_start(n, n_batches, b + k);
             ctd::RequestDesc &q = descs[static_cast<size_t>(b) * n_req + r];
             fill_request(P, seeds[r], q);
+            ctd::SharedTables sh{};
+            fill_shared(P, sh);
+            const LaunchShape one = launch_shape(ctx, sh, q.mode, false);
             set_range(q, n, n_batches, h0, h1, tallies[r], ctx->shared_launch ? 0 : static_cast<uint32_t>(nv), ctx->chunk,
-                      ctx->num_sms * ctx->threads / 32 *
-                          (ctx->shared_launch ? ctx->multi_blocks_per_sm : ctx->blocks_per_sm));
+                      ctx->shared_launch ? ctx->num_sms * ctx->multi_blocks_per_sm * ctx->threads / 32
+                                         : one.grid * (one.block / 32));
             q.work = ctx->u_work.p + static_cast<size_t>(b) * n_req + r;
             ctd::FoldDesc &f = folds[static_cast<size_t>(b) * n_req + r];
             f.tally = P.tally.p;
@@ -433,7 +436,10 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
     q.work = ctx->serve_work.p + R.lane;
     // batches of exactly B histories (of a problem that ends with these)
     const int nb = R.batches + std::max(n, 1);
-    const int warps = ctx->num_sms * ctx->blocks_per_sm * ctx->threads / 32;
+    ctd::SharedTables sh{};
+    fill_shared(P, sh);
+    const LaunchShape shape = launch_shape(ctx, sh, q.mode, false);
+    const int warps = shape.grid * (shape.block / 32);
     double hist = 0.0;
     for (int j = 0; j < std::max(n, 1); ++j) {
         const uint64_t first = static_cast<uint64_t>(R.batches + j) * B;

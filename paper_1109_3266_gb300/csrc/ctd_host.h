@@ -313,6 +313,11 @@ int join_lanes(ctd_ctx *ctx, cudaStream_t origin, int n);
 int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t s);
 // mean, standard error, avg RSD and deposited energy of nb finished batches
 int finish_stats(Phantom &P, int nb, cudaStream_t s);
+// grid, block and threads per SM of a single-request launch
+struct LaunchShape {
+    int grid, block, threads_per_sm;
+};
+LaunchShape launch_shape(const ctd_ctx *ctx, const ctd::SharedTables &sh, int mode, bool trace);
 // q covers histories [h0, h1) of the problem of n histories in nb batches, deposits of
 // its first batch into tally and of each later one `stride` voxels further on, for a
 // launch of `warps` warps

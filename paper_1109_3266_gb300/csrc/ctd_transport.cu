@@ -770,6 +770,8 @@ int launch_m(const LaunchParams &p, int grid, int block, int threads_per_sm, siz
              const L2Window *win)
 {
     // the register budget follows the residency asked for (65536 registers per SM)
+    if constexpr (kForm < 2)
+        if (block > 256) return launch_t<384, 3, kForm>(p, grid, block, smem, s, win);
     if (block <= 128 && threads_per_sm >= 896) return launch_t<128, 7, kForm>(p, grid, block, smem, s, win);
     if (threads_per_sm >= 1024) return launch_t<256, 4, kForm>(p, grid, block, smem, s, win);
     return launch_t<256, 3, kForm>(p, grid, block, smem, s, win);
@@ -788,13 +790,15 @@ size_t transport_smem_bytes(const LaunchParams &p, int threads)
 // persistent grids: a few blocks per SM
 constexpr int kMaxGrid = 1 << 16;
 
-// Kernel variants by residency: 4 blocks of 256 threads per SM cap it at 64
-// registers, 7 blocks of 128 at 73, fewer at 85.
+// Kernel variants by residency: 3 blocks of 384 threads per SM cap it at 56
+// registers, 4 of 256 at 64, 7 blocks of 128 at 73, fewer at 85.  Blocks of more than
+// 256 threads: full transport of one request, without records or wide indices.
 int launch_transport(const LaunchParams &p, int grid, int block, int threads_per_sm, void *stream,
                      const L2Window *win)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (grid <= 0 || grid > kMaxGrid || block <= 0 || block > 256 || block % 32 != 0) {
+    const bool large = p.n_req == 0 && !p.trace && !p.sh.wide && p.one.mode == CTD_MODE_FULL;
+    if (grid <= 0 || grid > kMaxGrid || block <= 0 || block > (large ? 384 : 256) || block % 32 != 0) {
         set_error("transport launch shape out of range");
         return CTD_EINVAL;
     }

@@ -61,3 +61,22 @@ def test_batched_chains_share_launches_like_plain_runs(ctd, contexts):
         assert [st[k] for k in COUNTS] == [t1[k] for k in COUNTS]
         assert np.allclose(dose, d1, rtol=1e-12, atol=0)
         ctd.ctd_destroy_phantom(c, h)
+
+
+@pytest.mark.parametrize("n_mat,e_max", [(1, 150), (16, 150), (16, 400), (16, 780)])
+def test_default_launch_shape_with_small_and_large_tables(ctd, contexts, n_mat, e_max):
+    # blocks of 384 threads while three of them fit beside the attenuation tables, else
+    # the 256-thread shape, up to tables that leave room for one block
+    rng = np.random.default_rng(5)
+    mats = [I.WATER, I.BONE, I.BRAIN, I.SOFT_TISSUE][:min(n_mat, 4)] * (4 if n_mat == 16 else 1)
+    shape = (16, 18, 20)
+    ph = I.Phantom(20, 18, 16, 0.5, 0.5, 0.5, rng.integers(0, n_mat, shape).astype(np.uint8),
+                   rng.uniform(0.5, 2.0, shape).astype(np.float32), mats)
+    p = I.Problem("tables", ph, I.arc_source(100.0, -4.0, 4.0, -3.0, 3.0, n_proj=90), I.spectrum_kramers(120, 2.5),
+                  I.Physics(e_max=e_max, n_zeta=64), 40_003, 3, 9)
+    explicit = ctd.ctd_create(device=0, threads_per_block=128, blocks_per_sm=1)
+    (d0, _, t0, h0), (d1, _, t1, _) = (ctd.run_problem(c, p) for c in (contexts[0], explicit))
+    ctd.ctd_destroy_phantom(contexts[0], h0)
+    ctd.ctd_destroy(explicit)
+    assert [t0[k] for k in COUNTS] == [t1[k] for k in COUNTS]
+    assert np.allclose(d0, d1, rtol=1e-12, atol=0)
