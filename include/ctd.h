@@ -567,7 +567,7 @@ int ctd_probe_memory(ctd_ctx *ctx, int kind, uint64_t n_slots, uint64_t n_ops, d
  * D > 0.1 D_max, rho >= 0.1 g/cm^3), [1] = the paper's sigma_bar, [2] = D_max,
  * written to 3 device doubles, asynchronously on stream (a cudaStream_t; NULL
  * is the legacy default stream).  No context is needed; it runs on the current
- * device.  It allocates nothing: its partial sums live in a fixed 160 KB
+ * device.  It allocates nothing: its partial sums live in a fixed 48 KB
  * device array inside the library, which every GPU that loads the library
  * holds until exit, so nvox may not exceed 67,108,864 (CTD_EINVAL beyond).
  * Each call looks up that array's device address on the current device (so a
