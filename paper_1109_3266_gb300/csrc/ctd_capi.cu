@@ -209,7 +209,7 @@ int ensure_run_buffers(Phantom &P)
     int rc;
     if ((rc = P.tally.ensure(P.nvox)) || (rc = P.sum_d.ensure(P.nvox)) || (rc = P.sum_d2.ensure(P.nvox)) ||
         (rc = P.edep.ensure(P.nvox)) || (rc = P.dose.ensure(P.nvox)) || (rc = P.sd.ensure(P.nvox)) ||
-        (rc = P.partials.ensure(6 * kRsdParts)) || (rc = P.result.ensure(8)) || (rc = P.counts.ensure(1)) ||
+        (rc = P.partials.ensure(ctd::kPartialDoubles)) || (rc = P.result.ensure(8)) || (rc = P.counts.ensure(1)) ||
         (rc = P.work.ensure(2)))
         return rc;
     return CTD_OK;
@@ -380,14 +380,27 @@ int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t
     return ctd::launch_transport(L, shape.grid, shape.block, shape.threads_per_sm, s);
 }
 
-// Mean, standard error, avg RSD and deposited energy of a finished run of nb
-// batches, on stream s.
+ctd::FoldLast last_of(Phantom &P, int nb, bool keep_sums)
+{
+    ctd::FoldLast l;
+    l.nb = nb;
+    l.inv_nb = 1.0 / nb;
+    l.inv_nn = 1.0 / (static_cast<double>(nb) * (nb - 1));
+    l.dose = P.dose.p;
+    l.sd = P.sd.p;
+    l.rho = P.rho.p;
+    l.partials = P.partials.p;
+    l.keep_sums = keep_sums;
+    return l;
+}
+
+// A last fold without batches, then the precision measures, on stream s.
 int finish_stats(Phantom &P, int nb, cudaStream_t s)
 {
-    int e = ctd::launch_finalize(P.sum_d.p, P.sum_d2.p, nb, P.dose.p, P.sd.p, P.nvox, s);
-    if (e == CTD_OK) e = ctd::launch_rsd(P.dose.p, P.sd.p, P.rho.p, P.nvox, P.partials.p, kRsdParts, P.result.p, s);
-    if (e == CTD_OK)
-        e = ctd::launch_sum(P.edep.p, P.nvox, P.partials.p + 5 * kRsdParts, kRsdParts, P.result.p + 3, s);
+    const ctd::FoldLast last = last_of(P, nb, false);
+    const ctd::FoldBatches none{};
+    int e = ctd::launch_fold(none, P.rinv.p, P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, false, &last, s);
+    if (e == CTD_OK) e = ctd::launch_rsd(last, P.nvox, P.result.p, s);
     return e;
 }
 
@@ -1022,10 +1035,8 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
     double *const tallies = group > 1 ? scratch.buf.p : P->tally.p;
     CK(cudaMemsetAsync(tallies, 0, nv * group * sizeof(double), ctx->stream));
     if (two) CK(cudaMemsetAsync(P->tally2.p, 0, nv * sizeof(double), ctx->stream));
-    CK(cudaMemsetAsync(P->sum_d.p, 0, nv * sizeof(double), ctx->stream));
-    CK(cudaMemsetAsync(P->sum_d2.p, 0, nv * sizeof(double), ctx->stream));
-    CK(cudaMemsetAsync(P->edep.p, 0, nv * sizeof(double), ctx->stream));
     CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+    const ctd::FoldLast last = last_of(*P, n_batches, false);
     ctd::RequestDesc T;
     fill_request(*P, seed, T);
     size_t launches = 0;
@@ -1040,7 +1051,7 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
                 return rc;
             ++launches;
             CKS(ctd::launch_fold(fold_of(*P, n_histories, n_batches, b, k, tallies, false), P->rinv.p, P->sum_d.p,
-                                 P->sum_d2.p, P->edep.p, nv, ctx->stream));
+                                 P->sum_d2.p, P->edep.p, nv, b == 0, b + k == n_batches ? &last : nullptr, ctx->stream));
         }
     } else {
         if (two) {
@@ -1060,16 +1071,14 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
                 return rc;
             if (two && b > 0) CK(cudaStreamWaitEvent(s, ctx->plain_fold[k ^ 1], 0));
             CKS(ctd::launch_fold(fold_of(*P, n_histories, n_batches, b, 1, tally, true), P->rinv.p, P->sum_d.p,
-                                 P->sum_d2.p, P->edep.p, nv, s));
+                                 P->sum_d2.p, P->edep.p, nv, b == 0, b + 1 == n_batches ? &last : nullptr, s));
             if (two) CK(cudaEventRecord(ctx->plain_fold[k], s));
         }
         launches = n_batches;
         // the context's stream continues after the last fold (which followed every other)
         if (two && ((n_batches - 1) & 1)) CK(cudaStreamWaitEvent(ctx->stream, ctx->plain_fold[1], 0));
     }
-    CKS(ctd::launch_finalize(P->sum_d.p, P->sum_d2.p, n_batches, P->dose.p, P->sd.p, nv, ctx->stream));
-    CKS(ctd::launch_rsd(P->dose.p, P->sd.p, P->rho.p, nv, P->partials.p, kRsdParts, P->result.p, ctx->stream));
-    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p + 5 * kRsdParts, kRsdParts, P->result.p + 3, ctx->stream));
+    CKS(ctd::launch_rsd(last, nv, P->result.p, ctx->stream));
     if ((rc = collect(ctx, *P, launches, t0))) return rc;
     scratch.idle = true;
     P->stats.histories = n_histories;
@@ -1106,7 +1115,7 @@ int ctd_run_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t s
         ++launches;
     }
     CK(cudaMemsetAsync(P->result.p, 0, 3 * sizeof(double), ctx->stream));
-    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p + 5 * kRsdParts, kRsdParts, P->result.p + 3, ctx->stream));
+    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p, P->result.p + 3, ctx->stream));
     if ((rc = collect(ctx, *P, launches, t0))) return rc;
     P->stats.histories = h_end - h_begin;
     P->stats.n_batches = n_batches;
@@ -1168,7 +1177,7 @@ int ctd_shard_fold(ctd_ctx *ctx, ctd_phantom ph, int batch, double *tally_dev)
     if (batch < 0 || batch >= P->shard_nb) return fail(CTD_EINVAL, "batch %d outside [0, %d)", batch, P->shard_nb);
     if (!tally_dev) return fail(CTD_EINVAL, "null tally buffer");
     CKS(ctd::launch_fold(fold_of(*P, P->shard_n, P->shard_nb, batch, 1, tally_dev, true), P->rinv.p, P->sum_d.p,
-                         P->sum_d2.p, P->edep.p, P->nvox, ctx->stream));
+                         P->sum_d2.p, P->edep.p, P->nvox, false, nullptr, ctx->stream));
     return CTD_OK;
 }
 
@@ -1250,7 +1259,7 @@ int ctd_trace_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t
         ++launches;
     }
     CK(cudaMemsetAsync(P->result.p, 0, 3 * sizeof(double), ctx->stream));
-    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p + 5 * kRsdParts, kRsdParts, P->result.p + 3, ctx->stream));
+    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p, P->result.p + 3, ctx->stream));
     if (n) CK(cudaMemcpyAsync(out, rec.p, n * sizeof(ctd_track), cudaMemcpyDeviceToHost, ctx->stream));
     if ((rc = collect(ctx, *P, launches, t0))) return rc;
     P->stats.histories = n;

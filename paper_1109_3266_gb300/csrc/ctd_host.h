@@ -205,8 +205,7 @@ struct ServeReq {
 
 // device memory a plain run may take, while it runs, for the tallies of batches that
 // share a launch, and a batched call for all its requests'
-constexpr size_t kTallyBudget = size_t(1) << 30, kBatchTallyBudget = size_t(512) << 20;
-constexpr int kRsdParts = 1024;   // partial sums of the statistics reductions
+constexpr size_t kTallyBudget = size_t(1) << 30, kBatchTallyBudget = size_t(2) << 30;
 constexpr int kMaxLanes = 64;     // streams for request chains
 constexpr uint64_t kMaxTrace = 1ull << 26;   // histories of one trace call (16 B of device memory each)
 
@@ -311,7 +310,9 @@ int fork_lanes(ctd_ctx *ctx, cudaStream_t origin, int n);
 int join_lanes(ctd_ctx *ctx, cudaStream_t origin, int n);
 // one single-request launch of q on stream s at the context's launch shape
 int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t s);
-// mean, standard error, avg RSD and deposited energy of nb finished batches
+// the last fold's outputs for a run of nb batches of P
+ctd::FoldLast last_of(Phantom &P, int nb, bool keep_sums);
+// mean, standard error, avg RSD and deposited energy of nb folded batches
 int finish_stats(Phantom &P, int nb, cudaStream_t s);
 // grid, block and threads per SM of a single-request launch
 struct LaunchShape {

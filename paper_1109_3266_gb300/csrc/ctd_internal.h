@@ -221,20 +221,35 @@ struct FoldBatches {
     int clear;
 };
 
+// The results of a fold that is a run's last: dose and standard error over nb batches
+// (inv_nb = 1/nb, inv_nn = 1/(nb (nb - 1))), and in `partials` (kPartialDoubles) what
+// launch_rsd goes on from.  keep_sums: the batch sums are stored too (more batches may
+// follow).
+struct FoldLast {
+    int nb;
+    double inv_nb, inv_nn;
+    double *dose, *sd;
+    const float *rho;
+    double *partials;
+    int keep_sums;
+};
+// partials: per block the largest dose, the deposited energy and four sums, then a counter
+constexpr int kPartialCells = 6 * 152 * 8, kPartialDoubles = kPartialCells + 1;
+
 // launches (ctd_transport.cu / ctd_stats.cu); win may be null
 int launch_transport(const LaunchParams &p, int grid, int block, int threads_per_sm, void *stream,
                      const L2Window *win = nullptr);
 size_t transport_smem_bytes(const LaunchParams &p, int threads);
+// fold of f's batches (f.nb may be 0); first: the sums start with them; last (may be
+// null): and the dose and its standard error follow
 int launch_fold(const FoldBatches &f, const double *rinv, double *sum_d, double *sum_d2, double *edep, size_t nvox,
-                void *stream);
-int launch_finalize(const double *sum_d, const double *sum_d2, int nb, double *dose, double *sd, size_t nvox,
-                    void *stream);
-int launch_rsd(const double *dose, const double *sd, const float *rho, size_t nvox, double *partials,
-               int n_parts, double *result, void *stream);
+                bool first, const FoldLast *last, void *stream);
+// result[0..3] = avg RSD, sigma-bar, D_max, deposited energy after a last fold
+int launch_rsd(const FoldLast &last, size_t nvox, double *result, void *stream);
 int launch_sample_mu(const float *surf, int n_zeta, int n_e, int e_min, float e, uint64_t seed, uint64_t n,
                      double *out, void *stream);
 int launch_eval_math(int fn, const float *x, float *out, size_t n, void *stream);
-int launch_sum(const double *x, size_t n, double *partials, int n_parts, double *result, void *stream);
+int launch_sum(const double *x, size_t n, double *partials, double *result, void *stream);
 
 // one fold over several requests' grids in a single launch; tiles of
 // kFoldTile voxels, tile_off[r] = first tile of request r

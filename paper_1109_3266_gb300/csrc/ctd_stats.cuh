@@ -7,12 +7,16 @@
 
 #include <cstddef>
 
+#include "ctd_internal.h"
+
 namespace ctd {
 namespace stats {
 
 constexpr int kThreads = 256;
 constexpr int kMaxStatBlocks = 152 * 8;   // resident blocks of 256 threads
 constexpr int kPerThread = 4;             // voxels a thread holds in flight
+
+static_assert(kPartialCells == 6 * kMaxStatBlocks, "six partials per block");
 
 inline int stat_blocks(size_t n, int per_thread)
 {
