@@ -4,12 +4,17 @@
 // the launch-shape search and the memory probes in ctd_tune.cu.
 #include <cuda_runtime.h>
 
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <thread>
 
 #include "ctd_host.h"
 
@@ -506,6 +511,88 @@ int prepare_run(ctd_ctx *ctx, Phantom &P, uint64_t n, int nb)
     if ((rc = build_tables(ctx, P))) return rc;
     if ((rc = upload_allocation(ctx, P, n, nb))) return rc;
     if ((rc = ensure_run_buffers(P))) return rc;
+    return CTD_OK;
+}
+
+// Device arrays read back into host memory the caller has just allocated: its pages
+// do not exist yet, and the copy itself (185 GB/s into existing pages) would wait for
+// the kernel to make them one by one, 4 ms for 134 MB.  A few threads make them, a
+// chunk at a time by writing one byte to each page of the destination (which the copy
+// overwrites), while the copies follow chunk by chunk.  Destinations that are small,
+// resident already (a reused or pinned buffer, by mincore) or not pageable memory are
+// copied as before.
+namespace {
+
+constexpr size_t kColdBytes = size_t(4) << 20, kReadChunk = size_t(8) << 20;
+
+// whether most of the n bytes at p are pages without memory behind them
+bool cold(const char *p, size_t n, size_t page)
+{
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p) & ~(page - 1);
+    const size_t pages = (reinterpret_cast<uintptr_t>(p) + n - a + page - 1) / page;
+    std::vector<unsigned char> in(pages);
+    if (mincore(reinterpret_cast<void *>(a), pages * page, in.data()) != 0) return false;
+    size_t there = 0;
+    for (unsigned char c : in) there += c & 1u;
+    return 2 * there < pages;
+}
+
+}  // namespace
+
+int read_back(ctd_ctx *ctx, const ReadPart *parts, int n_parts)
+{
+    struct Chunk {
+        char *dst;
+        const char *src;
+        size_t n;
+    };
+    const size_t page = static_cast<size_t>(sysconf(_SC_PAGESIZE));
+    size_t bytes = 0;
+    for (int i = 0; i < n_parts; ++i) bytes += parts[i].bytes;
+    std::vector<Chunk> chunks;
+    std::vector<std::thread> makers;
+    std::unique_ptr<std::atomic<int>[]> made;
+    std::atomic<size_t> next{0};
+    if (bytes >= kColdBytes) try {
+            bool any = false;
+            for (int i = 0; i < n_parts; ++i)
+                any = any || (parts[i].bytes >= page && cold(static_cast<char *>(parts[i].dst), parts[i].bytes, page));
+            if (any) {
+                for (int i = 0; i < n_parts; ++i)
+                    for (size_t o = 0; o < parts[i].bytes; o += kReadChunk)
+                        chunks.push_back({static_cast<char *>(parts[i].dst) + o, static_cast<const char *>(parts[i].src) + o,
+                                          std::min(kReadChunk, parts[i].bytes - o)});
+                made.reset(new std::atomic<int>[chunks.size()]());
+                const size_t hw = std::max(2u, std::thread::hardware_concurrency());
+                const size_t n = std::min({size_t(6), hw / 2, chunks.size()});
+                makers.reserve(n);
+                for (size_t t = 0; t < n; ++t)
+                    makers.emplace_back([&] {
+                        for (size_t k; (k = next.fetch_add(1)) < chunks.size();) {
+                            volatile char *p = chunks[k].dst;
+                            for (size_t o = 0; o < chunks[k].n; o += page) p[o] = 0;
+                            p[chunks[k].n - 1] = 0;
+                            made[k].store(1, std::memory_order_release);
+                        }
+                    });
+            }
+        } catch (const std::exception &) {
+            // no memory or no threads: what threads there are finish, the copies do not wait
+        }
+    cudaError_t e = cudaSuccess;
+    if (makers.empty()) {
+        for (int i = 0; i < n_parts && e == cudaSuccess; ++i)
+            e = cudaMemcpyAsync(parts[i].dst, parts[i].src, parts[i].bytes, cudaMemcpyDeviceToHost, ctx->stream);
+    } else {
+        for (size_t k = 0; k < chunks.size(); ++k) {
+            while (!made[k].load(std::memory_order_acquire)) std::this_thread::yield();
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(chunks[k].dst, chunks[k].src, chunks[k].n, cudaMemcpyDeviceToHost, ctx->stream);
+        }
+        for (std::thread &t : makers) t.join();
+    }
+    if (e != cudaSuccess) return fail(CTD_ECUDA, "cudaMemcpyAsync failed: %s", cudaGetErrorString(e));
+    CK(cudaStreamSynchronize(ctx->stream));
     return CTD_OK;
 }
 
@@ -1276,9 +1363,11 @@ int ctd_get_dose_and_stddev(ctd_ctx *ctx, ctd_phantom ph, double *dose, double *
     if (!P) return fail(CTD_ENOTFOUND, "unknown phantom %d", ph);
     if ((dose || stddev) && !P->have_result) return fail(CTD_EINVAL, "no completed ctd_run on this phantom");
     if ((dose || stddev) && nvox != P->nvox) return fail(CTD_EINVAL, "nvox %zu != phantom's %zu", nvox, P->nvox);
-    if (dose) CK(cudaMemcpyAsync(dose, P->dose.p, nvox * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    if (stddev) CK(cudaMemcpyAsync(stddev, P->sd.p, nvox * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    ReadPart parts[2];
+    int n = 0;
+    if (dose) parts[n++] = {dose, P->dose.p, nvox * sizeof(double)};
+    if (stddev) parts[n++] = {stddev, P->sd.p, nvox * sizeof(double)};
+    if ((rc = read_back(ctx, parts, n))) return rc;
     if (stats) *stats = P->stats;
     return CTD_OK;
 }
@@ -1291,9 +1380,8 @@ int ctd_get_edep(ctd_ctx *ctx, ctd_phantom ph, double *edep_kev, size_t nvox)
     if (!P) return fail(CTD_ENOTFOUND, "unknown phantom %d", ph);
     if (!edep_kev || nvox != P->nvox) return fail(CTD_EINVAL, "edep buffer must hold the phantom's voxels");
     if (!P->edep.p) return fail(CTD_EINVAL, "nothing has run on this phantom");
-    CK(cudaMemcpyAsync(edep_kev, P->edep.p, nvox * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    return CTD_OK;
+    const ReadPart part = {edep_kev, P->edep.p, nvox * sizeof(double)};
+    return read_back(ctx, &part, 1);
 }
 
 int ctd_get_tables(ctd_ctx *ctx, ctd_phantom ph, int *n_e, int *n_zeta, int *n_mat, double *mu_cum, double *mu_max,

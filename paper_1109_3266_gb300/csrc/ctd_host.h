@@ -346,6 +346,13 @@ ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, do
 int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1,
               double *tally, uint32_t stride, size_t ev_index, uint4 *trace = nullptr, uint64_t trace_h0 = 0,
               uint64_t trace_n = 0, cudaStream_t s = nullptr, unsigned long long *work = nullptr);
+// device arrays into host memory, waited for
+struct ReadPart {
+    void *dst;
+    const void *src;
+    size_t bytes;
+};
+int read_back(ctd_ctx *ctx, const ReadPart *parts, int n_parts);
 double now_s();
 int transport_time(ctd_ctx *ctx, size_t n_launch, double &t);
 // counts and results of several phantoms read back through pinned staging
