@@ -382,7 +382,7 @@ int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t
     L.chunk = ctx->chunk;
     L.flight_cap = ctx->flight_cap;
     const LaunchShape shape = launch_shape(ctx, L.sh, q.mode, false);
-    return ctd::launch_transport(L, shape.grid, shape.block, shape.threads_per_sm, s);
+    return launch_single(L, shape, s);
 }
 
 ctd::FoldLast last_of(Phantom &P, int nb, bool keep_sums)
@@ -432,20 +432,46 @@ LaunchShape launch_shape(const ctd_ctx *ctx, const ctd::SharedTables &sh, int mo
 // 32, one round of source photons.  1e6 histories (a 51x51x32 head, 183 per warp) took
 // 0.43 ms while half of them went in claims of 256, 0.24 in claims of 32; for 1e5 claims
 // of 18, so that every warp has one, took 0.080 ms, claims of 32 0.057.
+static void set_claims(ctd::RequestDesc &q, uint64_t h0, uint64_t h1, int chunk, int warps)
+{
+    const uint64_t larger = q.rem * (q.n_lo + 1);   // histories in the larger batches
+    q.b0 = static_cast<int>(h0 < larger ? h0 / (q.n_lo + 1) : q.rem + (h0 - larger) / q.n_lo);
+    q.h_begin = h0;
+    q.h_end = h1;
+    const uint64_t tail = 256 * static_cast<uint64_t>(std::max(warps, 1));
+    q.h_big = h1 - h0 > tail ? h1 - tail : h0;
+    q.small = std::min(32, chunk);
+    q.h_hi = static_cast<uint32_t>(h0 >> 32);
+    q.k0 = q.rk[0] ^ q.h_hi;
+}
+
 void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1, double *tally, uint32_t stride,
                int chunk, int warps)
 {
     q.n_lo = n / nb;
     q.rem = n % nb;
-    const uint64_t larger = q.rem * (q.n_lo + 1);   // histories in the larger batches
-    q.b0 = static_cast<int>(h0 < larger ? h0 / (q.n_lo + 1) : q.rem + (h0 - larger) / q.n_lo);
-    q.h_begin = h0;
-    q.h_end = h1;
-    const uint64_t w = static_cast<uint64_t>(std::max(warps, 1)), tail = 256 * w, count = h1 - h0;
-    q.h_big = count > tail ? h1 - tail : h0;
-    q.small = std::min(32, chunk);
     q.tally = tally;
     q.tally_stride = stride;
+    set_claims(q, h0, h1, chunk, warps);
+}
+
+int launch_single(ctd::LaunchParams &L, const LaunchShape &shape, cudaStream_t s, const ctd::L2Window *win)
+{
+    ctd::RequestDesc &q = L.one;
+    const uint64_t end = q.h_end;
+    double *const tally = q.tally;
+    const int b0 = q.b0, warps = shape.grid * (shape.block / 32);
+    for (uint64_t h = q.h_begin; h < end; h = q.h_end) {
+        const uint64_t last = h | 0xffffffffull;   // the last history with this upper word
+        if (h != q.h_begin || last < end - 1) {
+            if (h != q.h_begin && cudaMemsetAsync(q.work, 0, sizeof(unsigned long long), s) != cudaSuccess) return CTD_ECUDA;
+            set_claims(q, h, last < end - 1 ? last + 1 : end, L.chunk, warps);
+            q.tally = tally + static_cast<size_t>(q.b0 - b0) * q.tally_stride;
+        }
+        const int rc = ctd::launch_transport(L, shape.grid, shape.block, shape.threads_per_sm, s, win);
+        if (rc != CTD_OK) return rc;
+    }
+    return CTD_OK;
 }
 
 ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, double *tally, bool clear)
@@ -499,7 +525,7 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb,
         }
         win.hit_ratio = static_cast<float>(std::min(1.0, static_cast<double>(ctx->l2_setaside) / win.bytes));
     }
-    CKS(ctd::launch_transport(L, shape.grid, shape.block, shape.threads_per_sm, s, ctx->l2_persist ? &win : nullptr));
+    CKS(launch_single(L, shape, s, ctx->l2_persist ? &win : nullptr));
     CK(cudaEventRecord(e1, s));
     return CTD_OK;
 }

@@ -63,6 +63,61 @@ __device__ __forceinline__ U4 philox_rk(uint32_t c0, uint32_t c1, uint32_t c2, u
     return U4{c0, c1, c2, c3};
 }
 
+// Blocks (h, step, stream 0) of one history, for histories that share the upper word
+// of h.  Of the first two rounds' four products only M1 step and M0 times a word made
+// from it depend on the step; the others are the history's, kept as three words:
+//   a = lo(M0 h) ^ k1', b = hi(M1 c2) ^ k0', c = lo(M1 c2) with c2 = hi(M0 h) ^ k1
+// (k0, k1 the first round's keys, k0', k1' the second's).
+struct HistKey {
+    uint32_t a, b, c;
+};
+
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+
+// 1 / kPhiloxM0 modulo 2^32 (an odd number is its own inverse modulo 8; each step
+// doubles the bits that are right)
+constexpr uint32_t inverse32(uint32_t m)
+{
+    uint32_t x = m;
+    for (int i = 0; i < 4; ++i) x *= 2u - m * x;
+    return x;
+}
+constexpr uint32_t kPhiloxM0Inverse = inverse32(kPhiloxM0);
+static_assert(kPhiloxM0 * kPhiloxM0Inverse == 1u, "inverse modulo 2^32");
+
+__device__ __forceinline__ HistKey hist_key(uint32_t h, const uint32_t *rk)
+{
+    const uint64_t p0 = static_cast<uint64_t>(kPhiloxM0) * h;
+    const uint64_t p1 = static_cast<uint64_t>(kPhiloxM1) * (static_cast<uint32_t>(p0 >> 32) ^ rk[1]);
+    return HistKey{static_cast<uint32_t>(p0) ^ rk[3], static_cast<uint32_t>(p1 >> 32) ^ rk[2], static_cast<uint32_t>(p1)};
+}
+
+// the lower word of the history a key was made from
+__device__ __forceinline__ uint32_t hist_of(const HistKey &k, const uint32_t *rk)
+{
+    return (k.a ^ rk[3]) * kPhiloxM0Inverse;
+}
+
+// k0 is the first round's key ^ the upper word of h.  (The products are written as
+// 64-bit ones: the compiler then takes the fewest instructions, 112 per history on the
+// head against 117 with the high and low words apart.)
+__device__ __forceinline__ U4 philox_step(const HistKey &k, uint32_t step, uint32_t k0, const uint32_t *rk)
+{
+    const uint64_t s0 = static_cast<uint64_t>(kPhiloxM1) * step;
+    const uint64_t s1 = static_cast<uint64_t>(kPhiloxM0) * (static_cast<uint32_t>(s0 >> 32) ^ k0);
+    uint32_t c0 = k.b ^ static_cast<uint32_t>(s0), c1 = k.c;
+    uint32_t c2 = static_cast<uint32_t>(s1 >> 32) ^ k.a, c3 = static_cast<uint32_t>(s1);
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+        const uint64_t p0 = static_cast<uint64_t>(kPhiloxM0) * c0, p1 = static_cast<uint64_t>(kPhiloxM1) * c2;
+        c0 = static_cast<uint32_t>(p1 >> 32) ^ c1 ^ rk[2 * r];
+        c2 = static_cast<uint32_t>(p0 >> 32) ^ c3 ^ rk[2 * r + 1];
+        c1 = static_cast<uint32_t>(p1);
+        c3 = static_cast<uint32_t>(p0);
+    }
+    return U4{c0, c1, c2, c3};
+}
+
 __device__ __forceinline__ U4 block(uint64_t seed, uint64_t h, uint32_t step, uint32_t stream)
 {
     return philox(static_cast<uint32_t>(h), static_cast<uint32_t>(h >> 32), step, stream,

@@ -324,6 +324,9 @@ LaunchShape launch_shape(const ctd_ctx *ctx, const ctd::SharedTables &sh, int mo
 // launch of `warps` warps
 void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1, double *tally, uint32_t stride,
                int chunk, int warps);
+// launches L (one request, its range set) on s, in pieces whose histories share the
+// upper word of their index; the claim counter is at 0
+int launch_single(ctd::LaunchParams &L, const LaunchShape &shape, cudaStream_t s, const ctd::L2Window *win = nullptr);
 // batch b of n histories in nb batches: its first history
 inline uint64_t batch_start(uint64_t n, int nb, int b)
 {

@@ -115,6 +115,7 @@ struct alignas(16) RequestDesc {
     int b0;                      // batch of h_begin
     uint32_t tally_stride;       // voxels, or 0: every batch into one grid
     int small;
+    uint32_t h_hi, k0;           // single-request launches: upper word of every history's index, and ^ rk[0]
     int pad_;
     int n_mat;
     int nbins;

@@ -27,22 +27,35 @@ using namespace dev;
 struct Photon {
     float x, y, z;    // position in voxel units: (r - box origin) / voxel size per axis
     float ux, uy, uz, e;
-    uint64_t h;
-    uint32_t tally;   // first voxel of its batch's tally
+    uint64_t h;       // its history, in launches of several requests, else the history's
+    HistKey key;      // part of its random numbers
+    uint32_t tally;   // first voxel of its batch's tally (single-request launches)
     uint32_t step;
     int j;            // energy node of e, its fraction and 1 / the majorant there;
     float te, imax;   // they change only with e
 };
 
-// Philox block of (history, step, stream) of request q: the round keys are
-// taken from q when it sits in the kernel's parameter space (kKeys), else
-// derived from the seed.
-template <bool kKeys>
+// Philox block of (history, step, stream) of request q
 __device__ __forceinline__ U4 draw(const RequestDesc &q, uint64_t h, uint32_t step, uint32_t stream)
 {
-    if (kKeys)
-        return philox_rk(static_cast<uint32_t>(h), static_cast<uint32_t>(h >> 32), step, stream, q.rk);
-    return block(q.seed, h, step, stream);
+    return philox_rk(static_cast<uint32_t>(h), static_cast<uint32_t>(h >> 32), step, stream, q.rk);
+}
+
+// A transport block of a photon.  A single-request launch's histories share the upper
+// word of their index (the host splits a launch where it changes), so the photon
+// carries its history's part of the first two rounds: 18 products a block instead of
+// 20.  CBCT water 14.94 -> 14.58 ms per 2e8 histories, head 24.25 -> 24.07.
+template <bool kMulti>
+__device__ __forceinline__ U4 draw_step(const RequestDesc &q, const Photon &ph)
+{
+    return kMulti ? draw(q, ph.h, ph.step, kStreamTransport) : philox_step(ph.key, ph.step, q.k0, q.rk);
+}
+
+// the photon's history (for the records of a trace launch)
+template <bool kMulti>
+__device__ __forceinline__ uint64_t history(const RequestDesc &q, const Photon &ph)
+{
+    return kMulti ? ph.h : (static_cast<uint64_t>(q.h_hi) << 32) | hist_of(ph.key, q.rk);
 }
 
 // energy node, fraction and inverse majorant of the photon's energy
@@ -174,12 +187,12 @@ __device__ __forceinline__ int bin_search(const uint64_t *pref, int nbins, uint6
 // Source photon of history h of request q, history `local` of its batch, whose bin
 // starts are `pref`; `bin` is a lower bound of its 1 keV interval.  Returns true if the photon
 // enters the phantom.
-template <bool kKeys, bool kFluence, bool kTrace>
+template <bool kFluence, bool kTrace>
 __device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, const uint64_t *pref, uint64_t local, int bin,
                                        Photon &ph, LaneCounts &cnt, const Tracer &tr)
 {
     while (bin < q.nbins - 1 && __ldg(&pref[bin + 1]) <= local) ++bin;
-    const U4 b0 = draw<kKeys>(q, h, 0, kStreamSource);
+    const U4 b0 = draw(q, h, 0, kStreamSource);
     const float elo = __ldg(&q.bin_lo[bin]), ehi = __ldg(&q.bin_hi[bin]);
     const float e = __fmaf_rn(ehi - elo, uni(b0.x), elo);
     cnt.emitted(e);
@@ -204,7 +217,7 @@ __device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, const u
     bool accepted = false;
     float uu = 0.0f, vv = 0.0f, qq = 0.0f;
     if (kFluence && q.fl_n > 0) {
-        const U4 b = draw<kKeys>(q, h, 1, kStreamSource);
+        const U4 b = draw(q, h, 1, kStreamSource);
         const uint32_t k =
             static_cast<uint32_t>((static_cast<uint64_t>(b.x) * static_cast<uint64_t>(static_cast<uint32_t>(q.fl_n))) >> 32);
         const uint32_t beam = b.y < __ldg(&q.fl_thr[k]) ? k : static_cast<uint32_t>(__ldg(&q.fl_alias[k]));
@@ -216,7 +229,7 @@ __device__ __forceinline__ bool source(const RequestDesc &q, uint64_t h, const u
         accepted = true;
     }
     for (uint32_t t = 1; t <= kMaxTrials && !accepted; ++t) {
-        const U4 b = draw<kKeys>(q, h, t, kStreamSource);
+        const U4 b = draw(q, h, t, kStreamSource);
         uu = __fmaf_rn(q.uw, uni(b.x), q.ulo);
         vv = __fmaf_rn(q.vw, uni(b.y), q.vlo);
         qq = __fmaf_rn(vv, vv, __fmaf_rn(uu, uu, D2));
@@ -299,11 +312,11 @@ struct Site {
 // chain's waits with another's instructions.  With a branch per outcome CBCT water
 // took 16.70 ms of transport per 2e8 histories and the head 28.43; without,
 // 15.31 and 25.03 ms (bit-identical).
-template <bool kKeys, bool kWide>
+template <bool kMulti, bool kWide>
 __device__ __forceinline__ void flight(const SharedTables &sh, const RequestDesc &q, const float2 *__restrict__ s_tab,
                                        Photon &ph, Site &at)
 {
-    const U4 b = draw<kKeys>(q, ph.h, ph.step, kStreamTransport);
+    const U4 b = draw_step<kMulti>(q, ph);
     ph.step++;
     const float path = (-log32(uni(b.x))) * ph.imax;
     // the move in voxel units: each displacement s u_k times 1/d_k, added fused
@@ -359,7 +372,7 @@ __device__ __forceinline__ void flight(const SharedTables &sh, const RequestDesc
 // (CTD_MODE_MAX_REAL), where most histories end here and skip the rest; full
 // transport is compiled without that branch (with it 2 % slower on CBCT water, while
 // a primary-only run without it was 4 % slower).
-template <bool kWide, bool kAnyMode, bool kTrace>
+template <bool kMulti, bool kWide, bool kAnyMode, bool kTrace>
 __device__ __forceinline__ int interact(const SharedTables &sh, const RequestDesc &q, const float2 *__restrict__ s_tab,
                                         const float *__restrict__ s_mm, Photon &ph, const Site &at, LaneCounts &cnt,
                                         const Tracer &tr)
@@ -391,7 +404,7 @@ __device__ __forceinline__ int interact(const SharedTables &sh, const RequestDes
     const bool absorbed = pe || cutoff;
     ph.e = compton && !cutoff ? ec : e;
     const float dep = absorbed ? e : e - ph.e;
-    deposit(q.tally, at.idx + ph.tally, dep);
+    deposit(q.tally, kMulti ? at.idx : at.idx + ph.tally, dep);
     cnt.compton += compton;
     cnt.rayleigh += rayleigh;
     int end = pe ? kDonePe : cutoff ? kDoneCutoff : kNotEnded;
@@ -404,9 +417,10 @@ __device__ __forceinline__ int interact(const SharedTables &sh, const RequestDes
         rotate(ph.ux, ph.uy, ph.uz, mu, uni(at.rw));
     }
     if (kTrace) {
-        tr.last(ph.h, pe ? 0 : compton ? 1 : 2, at.idx);
+        const uint64_t h = history<kMulti>(q, ph);
+        tr.last(h, pe ? 0 : compton ? 1 : 2, at.idx);
         if (end != kNotEnded)
-            tr.end(ph.h, pe ? kEndPe : cutoff ? kEndCutoff : kEndTerminated, ph.step, dep);
+            tr.end(h, pe ? kEndPe : cutoff ? kEndCutoff : kEndTerminated, ph.step, dep);
     }
     return end;
 }
@@ -435,18 +449,20 @@ struct WarpPool {
 // took 9 % longer: the gathers' lines in flight need it).
 struct Queue {
     float4 *a;     // [kQueue] x, y, z (voxel units), ux
-    float4 *b;     // [kQueue] uy, uz, e, te
-    uint4 *c;      // [kQueue] h (lo, hi), first voxel of the batch's tally, bits of 1 / mu_max(e)
+    float4 *b;     // [kQueue] uy, uz, e, 1 / mu_max(e)
+    uint4 *c;      // [kQueue] the history's key and the first voxel of its batch's tally, or h (lo, hi)
     WarpPool *pool;
+    template <bool kMulti>
     __device__ __forceinline__ void put(int slot, const Photon &ph) const
     {
         a[slot] = make_float4(ph.x, ph.y, ph.z, ph.ux);
-        b[slot] = make_float4(ph.uy, ph.uz, ph.e, ph.te);
-        c[slot] = make_uint4(static_cast<uint32_t>(ph.h), static_cast<uint32_t>(ph.h >> 32), ph.tally,
-                             __float_as_uint(ph.imax));
+        b[slot] = make_float4(ph.uy, ph.uz, ph.e, ph.imax);
+        c[slot] = kMulti ? make_uint4(static_cast<uint32_t>(ph.h), static_cast<uint32_t>(ph.h >> 32), 0u, 0u)
+                         : make_uint4(ph.key.a, ph.key.b, ph.key.c, ph.tally);
     }
-    // all but the step; the node follows from e and te
-    __device__ __forceinline__ void get(int slot, Photon &ph, int e_min) const
+    // all but the step; the node follows from e
+    template <bool kMulti>
+    __device__ __forceinline__ void get(int slot, Photon &ph, const SharedTables &sh) const
     {
         const float4 u = a[slot], v = b[slot];
         const uint4 w = c[slot];
@@ -457,12 +473,14 @@ struct Queue {
         ph.uy = v.x;
         ph.uz = v.y;
         ph.e = v.z;
-        ph.te = v.w;
-        ph.h = w.x | (static_cast<uint64_t>(w.y) << 32);
-        ph.tally = w.z;
-        ph.imax = __uint_as_float(w.w);
-        // te = (e - e_min) - j exactly, so j is exact and this its bit pattern
-        ph.j = static_cast<int>(__float_as_uint(((ph.e - static_cast<float>(e_min)) - ph.te) + kTrunc) - kTruncBits);
+        ph.imax = v.w;
+        if (kMulti) {
+            ph.h = w.x | (static_cast<uint64_t>(w.y) << 32);
+        } else {
+            ph.key = HistKey{w.x, w.y, w.z};
+            ph.tally = w.w;
+        }
+        ph.j = enode(ph.e, sh.e_min, sh.n_e, ph.te);
     }
 };
 
@@ -480,7 +498,7 @@ static_assert(kWarpBytes % 16 == 0, "a warp's shared-memory area must keep 16-by
 // histories in 10 batches (32^3 water): 0.69 ms in 10 launches -> 0.071 in one; 1e6 in 7
 // (51x51x32 head) 2.83 -> 0.43; 1e7 in 10 (48x48x40 head, helix) 4.31 -> 1.47; 2e8 in 2
 // (CBCT water) 15.29 -> 15.00.
-template <bool kKeys, bool kFluence, bool kWide, bool kAnyMode, bool kTrace>
+template <bool kMulti, bool kFluence, bool kWide, bool kAnyMode, bool kTrace>
 __device__ __forceinline__ void run_request(const LaunchParams &P, const RequestDesc &q, const float2 *s_tab,
                                             const float *s_mm, const Queue &Q, int lane, LaneCounts &cnt)
 {
@@ -549,20 +567,23 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
                 // the lanes' own photons wait in the queue's free slots meanwhile, so that
                 // source sampling has the registers to itself
                 const int mine = qcount + lane;
-                Q.put(mine, ph);
+                Q.put<kMulti>(mine, ph);
                 __syncwarp();
                 Photon np;
                 bool ok = false;
                 if (lane < take)
-                    ok = source<kKeys, kFluence, kTrace>(q, next + lane, Q.pool->pref, next - Q.pool->first + lane,
+                    ok = source<kFluence, kTrace>(q, next + lane, Q.pool->pref, next - Q.pool->first + lane,
                                                          Q.pool->bin, np, cnt, tr);
                 const unsigned okm = __ballot_sync(kFull, ok);
-                Q.get(mine, ph, P.sh.e_min);
+                Q.get<kMulti>(mine, ph, P.sh);
                 __syncwarp();
                 if (ok) {
                     set_energy(np, P.sh, s_mm);
-                    np.tally = Q.pool->tally;
-                    Q.put(qcount + __popc(okm & lt_mask), np);
+                    if (!kMulti) {
+                        np.key = hist_key(static_cast<uint32_t>(np.h), q.rk);
+                        np.tally = Q.pool->tally;
+                    }
+                    Q.put<kMulti>(qcount + __popc(okm & lt_mask), np);
                 }
                 qcount += __popc(okm);
                 if (lane == 0) Q.pool->next = next + take;
@@ -576,7 +597,7 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
             const int rank = __popc(need & lt_mask);
             if (rank < npop) {
                 const int slot = qcount - 1 - rank;
-                Q.get(slot, ph, P.sh.e_min);
+                Q.get<kMulti>(slot, ph, P.sh);
                 ph.step = 0;
                 if (kAnyMode) cnt.me->nreal = 0;
                 alive = true;
@@ -596,18 +617,18 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
             if (ph.step + static_cast<uint32_t>(P.flight_cap) > kMaxSteps) lim = static_cast<int>(kMaxSteps - ph.step);
             if (lim == 0) {
                 end = kDoneAborted;
-                if (kTrace) tr.end(ph.h, kEndAborted, ph.step, 0.0f);
+                if (kTrace) tr.end(history<kMulti>(q, ph), kEndAborted, ph.step, 0.0f);
             } else {
                 Site at;
                 int k = 0;
                 do {
-                    flight<kKeys, kWide>(P.sh, q, s_tab, ph, at);
+                    flight<kMulti, kWide>(P.sh, q, s_tab, ph, at);
                 } while (at.fictitious && ++k < lim);
                 if (!at.inside) {
                     end = kDoneEscaped;
-                    if (kTrace) tr.end(ph.h, kEndEscaped, ph.step, 0.0f);
+                    if (kTrace) tr.end(history<kMulti>(q, ph), kEndEscaped, ph.step, 0.0f);
                 } else if (!at.fictitious) {
-                    end = interact<kWide, kAnyMode, kTrace>(P.sh, q, s_tab, s_mm, ph, at, cnt, tr);
+                    end = interact<kMulti, kWide, kAnyMode, kTrace>(P.sh, q, s_tab, s_mm, ph, at, cnt, tr);
                 }
             }
             // every way a history ends meets here, so that its lanes are counted together
@@ -670,7 +691,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) transport_kernel(cons
     if (!kMulti) {
         load_tables(P.one, n_e, s_tab, s_mm);
         __syncthreads();
-        run_request<true, kForm == 1, kWide, kAnyMode, kTrace>(P, P.one, reinterpret_cast<const float2 *>(s_tab), s_mm, Q, lane, cnt);
+        run_request<false, kForm == 1, kWide, kAnyMode, kTrace>(P, P.one, reinterpret_cast<const float2 *>(s_tab), s_mm, Q, lane, cnt);
         flush_warp(P.one.counts, cnt, Q.pool->sourced, lane);
         return;
     }

@@ -80,3 +80,29 @@ def test_default_launch_shape_with_small_and_large_tables(ctd, contexts, n_mat, 
     ctd.ctd_destroy(explicit)
     assert [t0[k] for k in COUNTS] == [t1[k] for k in COUNTS]
     assert np.allclose(d0, d1, rtol=1e-12, atol=0)
+
+
+HI = 1 << 32   # a launch's histories share the upper word of their index
+
+
+@pytest.mark.parametrize("a,b", [(HI - 3_000, HI + 2_000), (HI, HI + 1_000), (3 * HI - 1, 3 * HI + 1)])
+def test_histories_across_an_upper_word(ctd, contexts, oracle, a, b):
+    # records, counts and deposits of a range that a launch covers in two pieces, against
+    # the binary64 oracle and against the pieces run apart
+    from track_compare import compare
+
+    p = I.head(4 * HI + 5, 7, seed=21, shape=(32, 30, 20), d=0.8)
+    c = contexts[0]
+    h = ctd.load_problem(c, p)
+    dev = ctd.ctd_trace_range(c, h, p.n_hist, p.seed, p.n_batches, a, b)
+    s = compare(dev, oracle.Setup(p, 64).track(a, b, threads=16))
+    assert s["never_ended"] == 0 and s["mismatches"] <= 5e-3 * (b - a), s
+    whole, parts = [], []
+    for ranges, out in (([(a, b)], whole), ([(a, a + (b - a) // 3), (a + (b - a) // 3, b)], parts)):
+        for k, (lo, hi) in enumerate(ranges):
+            ctd.ctd_run_range(c, h, p.n_hist, p.seed, p.n_batches, lo, hi, clear=k == 0)
+        _, _, st = ctd.ctd_get_dose_and_stddev(c, h, 0, want_arrays=False)
+        out += [ctd.ctd_get_edep(c, h, p.phantom.nvox), [st[k] for k in COUNTS]]
+    ctd.ctd_destroy_phantom(c, h)
+    assert whole[1] == parts[1] and whole[1][-1] == int(dev["steps"].sum())
+    assert np.allclose(whole[0], parts[0], rtol=1e-12, atol=0)
