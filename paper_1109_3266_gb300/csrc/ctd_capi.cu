@@ -243,8 +243,7 @@ void fill_request(Phantom &P, uint64_t seed, ctd::RequestDesc &q)
     q.pref = P.pref.p;
     q.cs_stride = P.phys.compton_model == CTD_COMPTON_WH ? (P.n_e - 1) * (P.phys.n_zeta - 1) : 0;
     if (P.fl_nu > 0) {
-        q.fl_thr = P.fl_thr.p;
-        q.fl_alias = P.fl_alias.p;
+        q.fl = P.fl.p;
         q.fl_n = P.fl_nu * P.fl_nv;
         q.fl_nu = P.fl_nu;
         q.fl_magic = ((1ull << 40) / static_cast<uint64_t>(P.fl_nu)) + 1;
@@ -254,11 +253,8 @@ void fill_request(Phantom &P, uint64_t seed, ctd::RequestDesc &q)
     q.n_mat = static_cast<int>(P.mats.size());
     q.work = P.work.p;
     q.nbins = static_cast<int>(P.w.size());
-    q.bin_lo = P.bins.p;
-    q.bin_hi = P.bins.p + q.nbins;
-    q.cb = P.proj.p;
-    q.sb = P.proj.p + (P.src.n_proj > 0 ? P.src.n_proj : 1);
-    q.zb = P.proj.p + 2 * (P.src.n_proj > 0 ? P.src.n_proj : 1);
+    q.bins = P.bins.p;
+    q.proj = P.proj.p;
     q.hz0 = static_cast<float>(P.src.z0_cm);
     q.hdz = static_cast<float>(P.src.z1_cm - P.src.z0_cm);
     q.counts = P.counts.p;
@@ -937,17 +933,17 @@ int ctd_set_source(ctd_ctx *ctx, ctd_phantom ph, const ctd_source *src)
     if (src->kind == CTD_SRC_ARC && !src->continuous && (src->n_proj < 1 || src->n_proj > (1 << 24)))
         return fail(CTD_EINVAL, "n_proj must be 1..2^24");
     if (!std::isfinite(src->z0_cm) || !std::isfinite(src->z1_cm)) return fail(CTD_EINVAL, "source heights must be finite");
-    std::vector<float> tab(3 * np);
+    std::vector<float4> tab(np);
     for (int k = 0; k < np; ++k) {
         // projection angles b_k = arc0 + (arc1 - arc0) k / n_proj, heights z0 + (z1 - z0) k / n_proj
         const double b = src->arc0_rad + (src->arc1_rad - src->arc0_rad) * static_cast<double>(k) / static_cast<double>(np);
-        tab[k] = static_cast<float>(std::cos(b));
-        tab[np + k] = static_cast<float>(std::sin(b));
-        tab[2 * np + k] =
-            static_cast<float>(src->z0_cm + (src->z1_cm - src->z0_cm) * static_cast<double>(k) / static_cast<double>(np));
+        tab[k] = make_float4(
+            static_cast<float>(std::cos(b)), static_cast<float>(std::sin(b)),
+            static_cast<float>(src->z0_cm + (src->z1_cm - src->z0_cm) * static_cast<double>(k) / static_cast<double>(np)),
+            0.0f);
     }
     if ((rc = P->proj.ensure(tab.size()))) return rc;
-    CK(cudaMemcpyAsync(P->proj.p, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(P->proj.p, tab.data(), tab.size() * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     P->src = *src;
     P->src.n_proj = np;
@@ -973,9 +969,10 @@ int ctd_set_fluence(ctd_ctx *ctx, ctd_phantom ph, int n_u, int n_v, const double
     std::vector<int32_t> al(n);
     if (!ctd::alias_build(n, f, thr.data(), al.data()))
         return fail(CTD_EINVAL, "fluence map needs finite intensities >= 0 with a positive sum");
-    if ((rc = P->fl_thr.ensure(n)) || (rc = P->fl_alias.ensure(n))) return rc;
-    CK(cudaMemcpyAsync(P->fl_thr.p, thr.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(P->fl_alias.p, al.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
+    std::vector<uint2> cols(n);
+    for (int k = 0; k < n; ++k) cols[k] = make_uint2(thr[k], static_cast<unsigned>(al[k]));
+    if ((rc = P->fl.ensure(n))) return rc;
+    CK(cudaMemcpyAsync(P->fl.p, cols.data(), n * sizeof(uint2), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     P->h_thr.swap(thr);
     P->h_alias.swap(al);
@@ -1015,13 +1012,10 @@ int ctd_set_spectrum(ctd_ctx *ctx, ctd_phantom ph, const double *e_lo, const dou
     P->e_lo.assign(e_lo, e_lo + nbins);
     P->e_hi.assign(e_hi, e_hi + nbins);
     P->w.assign(w, w + nbins);
-    std::vector<float> b(2 * nbins);
-    for (int j = 0; j < nbins; ++j) {
-        b[j] = static_cast<float>(e_lo[j]);
-        b[nbins + j] = static_cast<float>(e_hi[j]);
-    }
+    std::vector<float2> b(nbins);
+    for (int j = 0; j < nbins; ++j) b[j] = make_float2(static_cast<float>(e_lo[j]), static_cast<float>(e_hi[j]));
     if ((rc = P->bins.ensure(b.size()))) return rc;
-    CK(cudaMemcpyAsync(P->bins.p, b.data(), b.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(P->bins.p, b.data(), b.size() * sizeof(float2), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     P->alloc_n = ~0ull;
     P->alloc_nb = -1;

@@ -129,8 +129,8 @@ struct Phantom {
     DevBuf<ctd::DeviceCounts> counts;
     DevBuf<unsigned long long> work;
     DevBuf<uint64_t> pref;     // [2][nbins+1]: batch of n_lo+1, batch of n_lo
-    DevBuf<float> bins;        // [2][nbins]: lo, hi
-    DevBuf<float> proj;        // [2][n_proj]: cos, sin
+    DevBuf<float2> bins;       // [nbins]: lo, hi
+    DevBuf<float4> proj;       // [n_proj]: cos, sin, height
     uint64_t alloc_n = ~0ull;
     int alloc_nb = -1;
     ctd_run_stats stats{};
@@ -140,8 +140,7 @@ struct Phantom {
     int fl_nu = 0, fl_nv = 0;
     std::vector<uint32_t> h_thr;
     std::vector<int32_t> h_alias;
-    DevBuf<uint32_t> fl_thr;
-    DevBuf<int32_t> fl_alias;
+    DevBuf<uint2> fl;          // threshold, alias
     // a sharded run in progress (ctd_shard_*): its history count, batches and seed
     uint64_t shard_n = 0, shard_seed = 0;
     int shard_nb = 0;
@@ -149,7 +148,10 @@ struct Phantom {
     // every device buffer of the phantom takes from and returns to cache c
     void use_cache(BufferCache *c)
     {
-        for (DevBuf<float> *b : {&rho, &tab, &mm, &cs, &rs, &bins, &proj}) b->cache = c;
+        for (DevBuf<float> *b : {&rho, &tab, &mm, &cs, &rs}) b->cache = c;
+        bins.cache = c;
+        proj.cache = c;
+        fl.cache = c;
         for (DevBuf<double> *b : {&tally, &tally2, &sum_d, &sum_d2, &edep, &dose, &sd, &partials, &result})
             b->cache = c;
         mat.cache = c;
@@ -158,8 +160,6 @@ struct Phantom {
         counts.cache = c;
         work.cache = c;
         pref.cache = c;
-        fl_thr.cache = c;
-        fl_alias.cache = c;
     }
 };
 

@@ -97,11 +97,8 @@ struct alignas(16) RequestDesc {
     const float *rsurf;          // [n_mat] surfaces of cells
     const float *csurf;          // [n_c] surfaces of cells, material m at m * cs_stride cells
     const uint64_t *pref;        // [2][nbins+1] bin starts inside a batch of n_lo + 1 and of n_lo histories
-    const float *bin_lo;         // [nbins]
-    const float *bin_hi;         // [nbins]
-    const float *cb;             // [n_proj]
-    const float *sb;             // [n_proj]
-    const float *zb;             // [n_proj] source height of each projection (helical)
+    const float2 *bins;          // [nbins] interval's low and high energy
+    const float4 *proj;          // [n_proj] cosine and sine of the angle, source height (helical), 0
     double *tally;               // [nvox] keV
     DeviceCounts *counts;
     unsigned long long *work;    // claim counter: histories claimed of [h_begin, h_end)
@@ -128,8 +125,7 @@ struct alignas(16) RequestDesc {
     float hz0, hdz;              // z0 and z1 - z0 of a continuous helical trajectory
     int mode, max_real;
     int cs_stride;               // 0 (one Klein-Nishina surface) or (n_e - 1)(n_zeta - 1) (Waller-Hartree)
-    const uint32_t *fl_thr;      // [fl_n] fluence-map alias thresholds (fl_n = 0: no map)
-    const int32_t *fl_alias;     // [fl_n]
+    const uint2 *fl;             // [fl_n] fluence-map alias threshold and alias (fl_n = 0: no map)
     int fl_n, fl_nu;
     float fl_du, fl_dv;          // beamlet size at the centre plane, cm
     uint64_t fl_magic;           // floor(2^40 / fl_nu) + 1: I / fl_nu = (I fl_magic) >> 40 for I < 2^24, fl_nu < 2^16
