@@ -616,18 +616,22 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
         if (alive) {
             // flights until a real interaction, the escape or flight_cap flights; then the
             // interaction.  A run stops short of the history's step limit; a history that
-            // has reached it is aborted when its next run would start.
-            int lim = P.flight_cap, end = kNotEnded;
-            if (ph.step + static_cast<uint32_t>(P.flight_cap) > kMaxSteps) lim = static_cast<int>(kMaxSteps - ph.step);
-            if (lim == 0) {
+            // has reached it is aborted when its next run would start.  The step count
+            // itself ends the loop (a counter beside it took head 23.62 instead of 23.19 ms
+            // per 2e8 histories, CBCT water 14.20 instead of 13.98), and the test for the
+            // limit stays in front of the loop: without an if around it the compiler let
+            // the lanes leave the loop one by one into the interaction (36.2 ms).
+            int end = kNotEnded;
+            const uint32_t capped = ph.step + static_cast<uint32_t>(P.flight_cap);
+            const uint32_t stop = capped < kMaxSteps ? capped : kMaxSteps;
+            if (ph.step >= kMaxSteps) {
                 end = kDoneAborted;
                 if (kTrace) tr.end(history<kMulti>(q, ph), kEndAborted, ph.step, 0.0f);
             } else {
                 Site at;
-                int k = 0;
                 do {
                     flight<kMulti, kWide>(P.sh, q, s_tab, ph, at);
-                } while (at.fictitious && ++k < lim);
+                } while (at.fictitious && ph.step < stop);
                 if (!at.inside) {
                     end = kDoneEscaped;
                     if (kTrace) tr.end(history<kMulti>(q, ph), kEndEscaped, ph.step, 0.0f);
