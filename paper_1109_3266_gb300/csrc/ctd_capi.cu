@@ -79,28 +79,6 @@ const std::vector<float> &angular_surface(ctd_ctx *ctx, int kind, double q0, con
     return ctx->surfaces.emplace(key, std::move(f)).first->second;
 }
 
-// Surfaces [k][n_e][n_zeta] as cells [k][n_e - 1][n_zeta - 1][4]: the corners
-// S[j][i], S[j][i+1], S[j+1][i], S[j+1][i+1] of the bilinear lookup in cell (j, i)
-static std::vector<float> surface_cells(const std::vector<float> &rows, int n_e, int n_zeta)
-{
-    const size_t row = static_cast<size_t>(n_e) * n_zeta;
-    const size_t cells = static_cast<size_t>(n_e - 1) * (n_zeta - 1);
-    const size_t k_max = rows.size() / row;
-    std::vector<float> out(k_max * cells * 4);
-    for (size_t k = 0; k < k_max; ++k)
-        for (int j = 0; j + 1 < n_e; ++j)
-            for (int i = 0; i + 1 < n_zeta; ++i) {
-                const float *r0 = &rows[k * row + static_cast<size_t>(j) * n_zeta + i];
-                const float *r1 = r0 + n_zeta;
-                float *o = &out[((k * (n_e - 1) + j) * (n_zeta - 1) + i) * 4];
-                o[0] = r0[0];
-                o[1] = r0[1];
-                o[2] = r1[0];
-                o[3] = r1[1];
-            }
-    return out;
-}
-
 // One material's node-table columns, from the context's cache
 static const std::vector<double> &material_columns(ctd_ctx *ctx, const ctd_material &mat, const ctd::Elements &el,
                                                    int e_min, int n_e, int compton_model)
@@ -161,12 +139,14 @@ int build_tables(ctd_ctx *ctx, Phantom &P)
                                           : angular_surface(ctx, 1, P.mats[m].q0, nullptr, ph.e_min_kev, n_e, ph.n_zeta);
         std::copy(r.begin(), r.end(), P.h_rs.begin() + m * row);
     }
-    // the device holds each surface as cells of the four corners of a bilinear lookup
-    const std::vector<float> cs_cells = surface_cells(P.h_cs, n_e, ph.n_zeta);
-    const std::vector<float> rs_cells = surface_cells(P.h_rs, n_e, ph.n_zeta);
+    // the device holds each surface as cells of the four corners of a bilinear lookup and
+    // makes them from the uploaded rows (a fourth of the bytes)
+    const size_t n_c = P.h_cs.size() / row, cells = static_cast<size_t>(n_e - 1) * (ph.n_zeta - 1) * 4;
+    DevBuf<float> rows;
+    rows.cache = &ctx->buffers;
     int rc;
-    if ((rc = P.tab.ensure(P.h_tab.size())) || (rc = P.mm.ensure(n_e)) || (rc = P.cs.ensure(cs_cells.size())) ||
-        (rc = P.rs.ensure(rs_cells.size())))
+    if ((rc = P.tab.ensure(P.h_tab.size())) || (rc = P.mm.ensure(n_e)) || (rc = P.cs.ensure(n_c * cells)) ||
+        (rc = P.rs.ensure(nm * cells)) || (rc = rows.ensure((n_c + nm) * row)))
         return rc;
     // on the device the two columns every step reads (total share, its difference) and
     // the two only a real interaction reads lie in separate planes
@@ -179,9 +159,12 @@ int build_tables(ctd_ctx *ctx, Phantom &P)
     }
     CK(cudaMemcpyAsync(P.tab.p, planes.data(), planes.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(P.mm.p, P.h_mm.data(), n_e * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(P.cs.p, cs_cells.data(), cs_cells.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(P.rs.p, rs_cells.data(), rs_cells.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(rows.p, P.h_cs.data(), n_c * row * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(rows.p + n_c * row, P.h_rs.data(), nm * row * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    const int rc_c = ctd::launch_cells(rows.p, static_cast<int>(n_c), n_e, ph.n_zeta, P.cs.p, ctx->stream);
+    const int rc_r = ctd::launch_cells(rows.p + n_c * row, nm, n_e, ph.n_zeta, P.rs.p, ctx->stream);
     CK(cudaStreamSynchronize(ctx->stream));
+    if (rc_c != CTD_OK || rc_r != CTD_OK) return fail(CTD_ECUDA, "launching the surface cells failed");
     P.n_e = n_e;
     P.tables_ok = true;
     return CTD_OK;

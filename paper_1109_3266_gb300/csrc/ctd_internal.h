@@ -243,6 +243,8 @@ int launch_fold(const FoldBatches &f, const double *rinv, double *sum_d, double 
                 bool first, const FoldLast *last, void *stream);
 // result[0..3] = avg RSD, sigma-bar, D_max, deposited energy after a last fold
 int launch_rsd(const FoldLast &last, size_t nvox, double *result, void *stream);
+// surfaces [k][n_e][n_zeta] as cells [k][n_e - 1][n_zeta - 1][4]
+int launch_cells(const float *rows, int k, int n_e, int n_zeta, float *cells, void *stream);
 int launch_sample_mu(const float *surf, int n_zeta, int n_e, int e_min, float e, uint64_t seed, uint64_t n,
                      double *out, void *stream);
 int launch_eval_math(int fn, const float *x, float *out, size_t n, void *stream);

@@ -216,6 +216,19 @@ __global__ void scan_phantom_kernel(const uint8_t *__restrict__ mat, const float
     }
 }
 
+// Angular surfaces [k][n_e][n_zeta] as cells [k][n_e - 1][n_zeta - 1] of float4: the
+// corners S[j][i], S[j][i+1], S[j+1][i], S[j+1][i+1] of the bilinear lookup in cell
+// (j, i).  One block per row of cells at a time; bound by the 16 bytes a cell written.
+__global__ void cells_kernel(const float *__restrict__ rows, int n_rows, int n_e, int n_zeta, float4 *__restrict__ cells)
+{
+    for (int r = blockIdx.x; r < n_rows; r += gridDim.x) {
+        const int m = r / (n_e - 1), j = r - m * (n_e - 1);
+        const float *r0 = rows + (static_cast<size_t>(m) * n_e + j) * n_zeta, *r1 = r0 + n_zeta;
+        float4 *out = cells + static_cast<size_t>(r) * (n_zeta - 1);
+        for (int i = threadIdx.x; i + 1 < n_zeta; i += blockDim.x) out[i] = make_float4(r0[i], r0[i + 1], r1[i], r1[i + 1]);
+    }
+}
+
 inline int ok() { return cudaGetLastError() == cudaSuccess ? CTD_OK : CTD_ECUDA; }
 
 }  // namespace
@@ -258,6 +271,14 @@ int launch_scan_phantom(const uint8_t *mat, const float *rho, size_t nvox, int n
     init.first_bad_rho = ~0ull;
     if (cudaMemcpyAsync(out, &init, sizeof(init), cudaMemcpyHostToDevice, s) != cudaSuccess) return CTD_ECUDA;
     scan_phantom_kernel<<<stat_blocks(nvox, 1), kThreads, 0, s>>>(mat, rho, nvox, n_mat, vox, rinv, out);
+    return ok();
+}
+
+int launch_cells(const float *rows, int k, int n_e, int n_zeta, float *cells, void *stream)
+{
+    const int n_rows = k * (n_e - 1);
+    cells_kernel<<<n_rows < kMaxStatBlocks ? n_rows : kMaxStatBlocks, kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
+        rows, n_rows, n_e, n_zeta, reinterpret_cast<float4 *>(cells));
     return ok();
 }
 
