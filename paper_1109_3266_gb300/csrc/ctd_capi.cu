@@ -197,8 +197,7 @@ int ensure_run_buffers(Phantom &P)
     int rc;
     if ((rc = P.tally.ensure(P.nvox)) || (rc = P.sum_d.ensure(P.nvox)) || (rc = P.sum_d2.ensure(P.nvox)) ||
         (rc = P.edep.ensure(P.nvox)) || (rc = P.dose.ensure(P.nvox)) || (rc = P.sd.ensure(P.nvox)) ||
-        (rc = P.partials.ensure(ctd::kPartialDoubles)) || (rc = P.result.ensure(8)) || (rc = P.counts.ensure(1)) ||
-        (rc = P.work.ensure(2)))
+        (rc = P.partials.ensure(ctd::kPartialDoubles)) || (rc = P.state.ensure(1)))
         return rc;
     return CTD_OK;
 }
@@ -234,13 +233,13 @@ void fill_request(Phantom &P, uint64_t seed, ctd::RequestDesc &q)
         q.fl_dv = static_cast<float>((P.src.v_hi_cm - P.src.v_lo_cm) / static_cast<double>(P.fl_nv));
     }
     q.n_mat = static_cast<int>(P.mats.size());
-    q.work = P.work.p;
+    q.work = P.work();
     q.nbins = static_cast<int>(P.w.size());
     q.bins = P.bins.p;
     q.proj = P.proj.p;
     q.hz0 = static_cast<float>(P.src.z0_cm);
     q.hdz = static_cast<float>(P.src.z1_cm - P.src.z0_cm);
-    q.counts = P.counts.p;
+    q.counts = P.counts();
     q.seed = seed;
     q.nx = P.nx;
     q.ny = P.ny;
@@ -384,7 +383,7 @@ int finish_stats(Phantom &P, int nb, cudaStream_t s)
     const ctd::FoldLast last = last_of(P, nb, false);
     const ctd::FoldBatches none{};
     int e = ctd::launch_fold(none, P.rinv.p, P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, false, &last, s);
-    if (e == CTD_OK) e = ctd::launch_rsd(last, P.nvox, P.result.p, s);
+    if (e == CTD_OK) e = ctd::launch_rsd(last, P.nvox, P.result(), s);
     return e;
 }
 
@@ -470,10 +469,10 @@ ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, do
 
 int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1,
               double *tally, uint32_t stride, size_t ev_index, uint4 *trace, uint64_t trace_h0, uint64_t trace_n,
-              cudaStream_t s, unsigned long long *work)
+              cudaStream_t s, unsigned long long *work, bool clear_work)
 {
     if (!s) s = ctx->stream;
-    if (!work) work = P.work.p;
+    if (!work) work = P.work();
     ctd::LaunchParams L;
     std::memset(&L, 0, sizeof(L));
     L.trace = trace;
@@ -486,7 +485,7 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb,
     L.one = q;
     L.chunk = ctx->chunk;
     L.flight_cap = ctx->flight_cap;
-    CK(cudaMemsetAsync(work, 0, sizeof(unsigned long long), s));
+    if (clear_work) CK(cudaMemsetAsync(work, 0, sizeof(unsigned long long), s));
     cudaEvent_t e0 = event_at(ctx, 2 * ev_index), e1 = event_at(ctx, 2 * ev_index + 1);
     if (!e0 || !e1) return fail(CTD_ECUDA, "cudaEventCreate failed");
     CK(cudaEventRecord(e0, s));
@@ -628,18 +627,14 @@ int collect_many(ctd_ctx *ctx, Phantom *const *ps, int n, size_t n_launch, doubl
         if (ctx->staged) cudaFreeHost(ctx->staged);
         ctx->staged = nullptr;
         ctx->staged_n = 0;
-        if (cudaMallocHost(reinterpret_cast<void **>(&ctx->staged), n * sizeof(Staged)) != cudaSuccess) {
+        if (cudaMallocHost(reinterpret_cast<void **>(&ctx->staged), n * sizeof(ctd::RunState)) != cudaSuccess) {
             cudaGetLastError();
             return fail(CTD_ENOMEM, "cudaMallocHost failed");
         }
         ctx->staged_n = n;
     }
-    for (int i = 0; i < n; ++i) {
-        CK(cudaMemcpyAsync(&ctx->staged[i].c, ps[i]->counts.p, sizeof(ctd::DeviceCounts), cudaMemcpyDeviceToHost,
-                           cs));
-        CK(cudaMemcpyAsync(ctx->staged[i].res, ps[i]->result.p, sizeof(ctx->staged[i].res), cudaMemcpyDeviceToHost,
-                           cs));
-    }
+    for (int i = 0; i < n; ++i)
+        CK(cudaMemcpyAsync(&ctx->staged[i], ps[i]->state.p, sizeof(ctd::RunState), cudaMemcpyDeviceToHost, cs));
     CK(cudaStreamSynchronize(cs));
     const double t_now = now_s();
     double t_transport;
@@ -647,7 +642,7 @@ int collect_many(ctd_ctx *ctx, Phantom *const *ps, int n, size_t n_launch, doubl
     if ((rc = transport_time(ctx, n_launch, t_transport))) return rc;
     for (int i = 0; i < n; ++i) {
         const ctd::DeviceCounts &c = ctx->staged[i].c;
-        const double *res = ctx->staged[i].res;
+        const double *res = ctx->staged[i].result;
         ctd_run_stats &s = ps[i]->stats;
         s.pe = c.n[ctd::kCntPe];
         s.compton = c.n[ctd::kCntCompton];
@@ -1125,7 +1120,7 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
     double *const tallies = group > 1 ? scratch.buf.p : P->tally.p;
     CK(cudaMemsetAsync(tallies, 0, nv * group * sizeof(double), ctx->stream));
     if (two) CK(cudaMemsetAsync(P->tally2.p, 0, nv * sizeof(double), ctx->stream));
-    CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+    CK(cudaMemsetAsync(P->state.p, 0, sizeof(ctd::RunState), ctx->stream));
     const ctd::FoldLast last = last_of(*P, n_batches, false);
     ctd::RequestDesc T;
     fill_request(*P, seed, T);
@@ -1137,7 +1132,8 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
             const int k = std::min(group, n_batches - b);
             if (b > 0) CK(cudaMemsetAsync(tallies, 0, nv * k * sizeof(double), ctx->stream));
             if ((rc = transport(ctx, *P, T, n_histories, n_batches, batch_start(n_histories, n_batches, b),
-                                batch_start(n_histories, n_batches, b + k), tallies, static_cast<uint32_t>(nv), launches)))
+                                batch_start(n_histories, n_batches, b + k), tallies, static_cast<uint32_t>(nv), launches,
+                                nullptr, 0, 0, nullptr, nullptr, b > 0)))
                 return rc;
             ++launches;
             CKS(ctd::launch_fold(fold_of(*P, n_histories, n_batches, b, k, tallies, false), P->rinv.p, P->sum_d.p,
@@ -1157,7 +1153,7 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
             const cudaStream_t s = k ? ctx->plain_aux : ctx->stream;
             double *tally = k ? P->tally2.p : P->tally.p;
             if ((rc = transport(ctx, *P, T, n_histories, n_batches, batch_start(n_histories, n_batches, b),
-                                batch_start(n_histories, n_batches, b + 1), tally, 0, b, nullptr, 0, 0, s, P->work.p + k)))
+                                batch_start(n_histories, n_batches, b + 1), tally, 0, b, nullptr, 0, 0, s, P->work() + k)))
                 return rc;
             if (two && b > 0) CK(cudaStreamWaitEvent(s, ctx->plain_fold[k ^ 1], 0));
             CKS(ctd::launch_fold(fold_of(*P, n_histories, n_batches, b, 1, tally, true), P->rinv.p, P->sum_d.p,
@@ -1168,7 +1164,7 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
         // the context's stream continues after the last fold (which followed every other)
         if (two && ((n_batches - 1) & 1)) CK(cudaStreamWaitEvent(ctx->stream, ctx->plain_fold[1], 0));
     }
-    CKS(ctd::launch_rsd(last, nv, P->result.p, ctx->stream));
+    CKS(ctd::launch_rsd(last, nv, P->result(), ctx->stream));
     if ((rc = collect(ctx, *P, launches, t0))) return rc;
     scratch.idle = true;
     P->stats.histories = n_histories;
@@ -1193,7 +1189,7 @@ int ctd_run_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t s
     const size_t nv = P->nvox;
     if (clear) {
         CK(cudaMemsetAsync(P->edep.p, 0, nv * sizeof(double), ctx->stream));
-        CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+        CK(cudaMemsetAsync(P->counts(), 0, sizeof(ctd::DeviceCounts), ctx->stream));
     }
     P->have_result = false;
     ctd::RequestDesc T;
@@ -1204,8 +1200,8 @@ int ctd_run_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t s
         if ((rc = transport(ctx, *P, T, n_histories, n_batches, h_begin, h_end, P->edep.p, 0, launches))) return rc;
         ++launches;
     }
-    CK(cudaMemsetAsync(P->result.p, 0, 3 * sizeof(double), ctx->stream));
-    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p, P->result.p + 3, ctx->stream));
+    CK(cudaMemsetAsync(P->result(), 0, 3 * sizeof(double), ctx->stream));
+    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p, P->result() + 3, ctx->stream));
     if ((rc = collect(ctx, *P, launches, t0))) return rc;
     P->stats.histories = h_end - h_begin;
     P->stats.n_batches = n_batches;
@@ -1226,7 +1222,7 @@ int ctd_shard_begin(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t
     CK(cudaMemsetAsync(P->sum_d.p, 0, nv * sizeof(double), ctx->stream));
     CK(cudaMemsetAsync(P->sum_d2.p, 0, nv * sizeof(double), ctx->stream));
     CK(cudaMemsetAsync(P->edep.p, 0, nv * sizeof(double), ctx->stream));
-    CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+    CK(cudaMemsetAsync(P->counts(), 0, sizeof(ctd::DeviceCounts), ctx->stream));
     P->have_result = false;
     P->shard_n = n_histories;
     P->shard_nb = n_batches;
@@ -1279,7 +1275,7 @@ int ctd_shard_counts(ctd_ctx *ctx, ctd_phantom ph, uint64_t *counts, double *ene
     if (!P) return fail(CTD_ENOTFOUND, "unknown phantom %d", ph);
     if (!counts || !energies) return fail(CTD_EINVAL, "null output");
     ctd::DeviceCounts c;
-    CK(cudaMemcpyAsync(&c, P->counts.p, sizeof(c), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(&c, P->counts(), sizeof(c), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     for (int i = 0; i < 10; ++i) counts[i] = c.n[i];
     energies[0] = ctd::fixed_kev(c.e_fix[0], c.e_fix[1]);
@@ -1338,7 +1334,7 @@ int ctd_trace_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t
     const size_t nv = P->nvox;
     CK(cudaMemsetAsync(rec.p, 0, (n ? n : 1) * sizeof(uint4), ctx->stream));
     CK(cudaMemsetAsync(P->edep.p, 0, nv * sizeof(double), ctx->stream));
-    CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+    CK(cudaMemsetAsync(P->counts(), 0, sizeof(ctd::DeviceCounts), ctx->stream));
     P->have_result = false;
     ctd::RequestDesc T;
     fill_request(*P, seed, T);
@@ -1348,8 +1344,8 @@ int ctd_trace_range(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t
         if ((rc = transport(ctx, *P, T, n_histories, n_batches, h_begin, h_end, P->edep.p, 0, launches, rec.p, h_begin, n))) return rc;
         ++launches;
     }
-    CK(cudaMemsetAsync(P->result.p, 0, 3 * sizeof(double), ctx->stream));
-    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p, P->result.p + 3, ctx->stream));
+    CK(cudaMemsetAsync(P->result(), 0, 3 * sizeof(double), ctx->stream));
+    CKS(ctd::launch_sum(P->edep.p, nv, P->partials.p, P->result() + 3, ctx->stream));
     if (n) CK(cudaMemcpyAsync(out, rec.p, n * sizeof(ctd_track), cudaMemcpyDeviceToHost, ctx->stream));
     if ((rc = collect(ctx, *P, launches, t0))) return rc;
     P->stats.histories = n;

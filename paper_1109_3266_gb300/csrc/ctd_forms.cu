@@ -91,7 +91,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             CK(cudaMemsetAsync(P.sum_d2.p, 0, nv * sizeof(double), ctx->stream));
             CK(cudaMemsetAsync(P.edep.p, 0, nv * sizeof(double), ctx->stream));
         }
-        CK(cudaMemsetAsync(P.counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+        CK(cudaMemsetAsync(P.counts(), 0, sizeof(ctd::DeviceCounts), ctx->stream));
         P.have_result = false;
         const uint64_t n = n_histories[r];
         const double vol = P.dx * P.dy * P.dz;
@@ -172,7 +172,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
                                              P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, b == 0,
                                              b + g == n_batches ? &last : nullptr, ls);
                 }
-                if (e == CTD_OK) e = ctd::launch_rsd(last, P.nvox, P.result.p, ls);
+                if (e == CTD_OK) e = ctd::launch_rsd(last, P.nvox, P.result(), ls);
             }
             if (e == CTD_OK) e = join_lanes(ctx, cs, n_lanes);
             if (e == CTD_OK && cudaEventRecordWithFlags(ctx->events[1], cs, cudaEventRecordExternal) != cudaSuccess)
@@ -236,7 +236,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     const void *work = ctx->u_work.p;
     put(&work, sizeof(work));
     for (int r = 0; r < n_req; ++r) {
-        const void *out[4] = {ps[r]->dose.p, ps[r]->sd.p, ps[r]->partials.p, ps[r]->result.p};
+        const void *out[4] = {ps[r]->dose.p, ps[r]->sd.p, ps[r]->partials.p, ps[r]->result()};
         put(out, sizeof(out));
     }
     // The batch loop is captured once into a CUDA graph and replayed while the
@@ -336,7 +336,7 @@ int clear_run(Phantom &P, cudaStream_t s)
     CK(cudaMemsetAsync(P.sum_d.p, 0, nv * sizeof(double), s));
     CK(cudaMemsetAsync(P.sum_d2.p, 0, nv * sizeof(double), s));
     CK(cudaMemsetAsync(P.edep.p, 0, nv * sizeof(double), s));
-    CK(cudaMemsetAsync(P.counts.p, 0, sizeof(ctd::DeviceCounts), s));
+    CK(cudaMemsetAsync(P.counts(), 0, sizeof(ctd::DeviceCounts), s));
     return CTD_OK;
 }
 
@@ -475,8 +475,8 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
         if (j == n - 2) CK(cudaEventRecord(ctx->serve_ev_pre[R.lane], s));
     }
     if (R.checked) {
-        CKS(ctd::launch_rsd(last, P.nvox, P.result.p, s));
-        CK(cudaMemcpyAsync(ctx->serve_res + 4 * R.lane, P.result.p, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
+        CKS(ctd::launch_rsd(last, P.nvox, P.result(), s));
+        CK(cudaMemcpyAsync(ctx->serve_res + 4 * R.lane, P.result(), 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
     }
     CK(cudaEventRecord(ctx->serve_ev[R.lane], s));
     R.group = n;
@@ -736,7 +736,7 @@ int serve_round(ctd_ctx *ctx)
     }
     std::vector<std::array<double, 3>> res(checked.size());
     for (size_t c = 0; c < checked.size(); ++c)
-        if (cudaMemcpyAsync(res[c].data(), ps[checked[c]]->result.p, 3 * sizeof(double), cudaMemcpyDeviceToHost,
+        if (cudaMemcpyAsync(res[c].data(), ps[checked[c]]->result(), 3 * sizeof(double), cudaMemcpyDeviceToHost,
                             ctx->stream) != cudaSuccess)
             return failed(fail(CTD_ECUDA, "served round: reading the statistics failed"));
     const cudaError_t se = cudaStreamSynchronize(ctx->stream);

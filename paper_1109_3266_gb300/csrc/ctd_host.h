@@ -124,10 +124,12 @@ struct Phantom {
     std::vector<float> h_tab, h_mm, h_cs, h_rs;
     DevBuf<float> tab, mm, cs, rs;
     // per-run state
-    DevBuf<double> tally, sum_d, sum_d2, edep, dose, sd, partials, result;
+    DevBuf<double> tally, sum_d, sum_d2, edep, dose, sd, partials;
     DevBuf<double> tally2;     // the second stream's batch tally of an overlapped plain run
-    DevBuf<ctd::DeviceCounts> counts;
-    DevBuf<unsigned long long> work;
+    DevBuf<ctd::RunState> state;
+    ctd::DeviceCounts *counts() const { return &state.p->c; }
+    unsigned long long *work() const { return state.p->work; }
+    double *result() const { return state.p->result; }
     DevBuf<uint64_t> pref;     // [2][nbins+1]: batch of n_lo+1, batch of n_lo
     DevBuf<float2> bins;       // [nbins]: lo, hi
     DevBuf<float4> proj;       // [n_proj]: cos, sin, height
@@ -152,13 +154,12 @@ struct Phantom {
         bins.cache = c;
         proj.cache = c;
         fl.cache = c;
-        for (DevBuf<double> *b : {&tally, &tally2, &sum_d, &sum_d2, &edep, &dose, &sd, &partials, &result})
+        for (DevBuf<double> *b : {&tally, &tally2, &sum_d, &sum_d2, &edep, &dose, &sd, &partials})
             b->cache = c;
         mat.cache = c;
         vox.cache = c;
         rinv.cache = c;
-        counts.cache = c;
-        work.cache = c;
+        state.cache = c;
         pref.cache = c;
     }
 };
@@ -174,11 +175,6 @@ struct Scratch {
     {
         if (buf.p && !idle) cudaStreamSynchronize(stream);
     }
-};
-
-struct Staged {
-    ctd::DeviceCounts c;
-    double res[4];    // avg RSD, sigma_bar, D_max, deposited energy
 };
 
 struct ServeReq {
@@ -259,7 +255,7 @@ struct ctd_ctx {
     cudaStream_t plain_aux = nullptr;
     cudaEvent_t plain_fork = nullptr, plain_fold[2] = {nullptr, nullptr};
     size_t l2_asked = 0, l2_setaside = 0, l2_persist_max = 0, l2_window_max = 0, l2_prev_limit = 0;
-    ctd::host::Staged *staged = nullptr;      // pinned read-back of counts and results
+    ctd::RunState *staged = nullptr;      // pinned read-back of counts and results
     size_t staged_n = 0;
     // angular surfaces by (kind, q0, e_min, n_e, n_zeta[, the elements' (Z, count) pairs]):
     // they do not depend on the phantom
@@ -345,10 +341,12 @@ ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, do
 // one transport launch over histories [h0, h1) of n in nb batches (set_range), bracketed
 // by timing events 2 ev_index and 2 ev_index + 1
 // (trace: per-history records of histories trace_h0 .. trace_h0 + trace_n - 1, or nullptr)
-// on stream s (null: the context's) with claim counter work (null: the phantom's first)
+// on stream s (null: the context's) with claim counter work (null: the phantom's first),
+// cleared here unless it is 0 already
 int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1,
               double *tally, uint32_t stride, size_t ev_index, uint4 *trace = nullptr, uint64_t trace_h0 = 0,
-              uint64_t trace_n = 0, cudaStream_t s = nullptr, unsigned long long *work = nullptr);
+              uint64_t trace_n = 0, cudaStream_t s = nullptr, unsigned long long *work = nullptr,
+              bool clear_work = true);
 // device arrays into host memory, waited for
 struct ReadPart {
     void *dst;

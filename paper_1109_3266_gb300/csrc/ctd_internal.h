@@ -74,6 +74,15 @@ struct DeviceCounts {
     unsigned long long e_fix[4];  // emitted lo, hi, escaped lo, hi: keV * 2^23 as 128-bit integers
 };
 
+// What a run of a phantom counts and reports, cleared by one memset and read back by
+// one copy: its counts, the claim counters of its launches, and avg RSD, sigma-bar,
+// D_max and the total deposit.
+struct RunState {
+    DeviceCounts c;
+    unsigned long long work[2];
+    double result[4];
+};
+
 // keV from a 128-bit fixed-point total (lo, hi) in units of 2^-23 keV
 inline double fixed_kev(unsigned long long lo, unsigned long long hi)
 {

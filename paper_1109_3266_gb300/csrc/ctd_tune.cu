@@ -90,7 +90,7 @@ int ctd_autotune(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_probe, uint64_t seed, 
         ctx->flight_cap = s.cap;
         t_min = 1e300;
         for (int rep = 0; rep < 2; ++rep) {
-            CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+            CK(cudaMemsetAsync(P->counts(), 0, sizeof(ctd::DeviceCounts), ctx->stream));
             int e;
             if ((e = transport(ctx, *P, q, P->alloc_n, P->alloc_nb, 0, n, P->tally.p, 0, 0))) return e;
             CK(cudaStreamSynchronize(ctx->stream));
@@ -143,7 +143,7 @@ int ctd_autotune(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_probe, uint64_t seed, 
         }
     }
     CK(cudaMemsetAsync(P->tally.p, 0, P->nvox * sizeof(double), ctx->stream));
-    CK(cudaMemsetAsync(P->counts.p, 0, sizeof(ctd::DeviceCounts), ctx->stream));
+    CK(cudaMemsetAsync(P->counts(), 0, sizeof(ctd::DeviceCounts), ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->threads = pick.threads;
     ctx->blocks_per_sm = pick.bps;
