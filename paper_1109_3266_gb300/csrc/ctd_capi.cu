@@ -1111,13 +1111,10 @@ int ctd_run(ctd_ctx *ctx, ctd_phantom ph, uint64_t n_histories, uint64_t seed, i
     if (two && (rc = ensure_plain_aux(ctx, *P))) return rc;
     // Batches that share a launch have a tally each, in scratch memory while the call
     // runs; without room for it (or where launches are per batch) the phantom's one.
-    Scratch scratch(&ctx->buffers, ctx->stream);
+    Scratch scratch(ctx->buffers, ctx->stream);
     int group = two || ctx->l2_persist ? 1 : tallies_within(nv, n_batches, kTallyBudget);
-    if (group > 1 && scratch.buf.ensure(nv * group)) {
-        g_error.clear();
-        group = 1;
-    }
-    double *const tallies = group > 1 ? scratch.buf.p : P->tally.p;
+    if (group > 1 && !scratch.borrow(nv * group)) group = 1;
+    double *const tallies = group > 1 ? scratch.p : P->tally.p;
     CK(cudaMemsetAsync(tallies, 0, nv * group * sizeof(double), ctx->stream));
     if (two) CK(cudaMemsetAsync(P->tally2.p, 0, nv * sizeof(double), ctx->stream));
     CK(cudaMemsetAsync(P->state.p, 0, sizeof(ctd::RunState), ctx->stream));

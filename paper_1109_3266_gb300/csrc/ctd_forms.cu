@@ -54,12 +54,13 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     // the larger grids' batches in launches of their own, 9.7 ms one ctd_run after another.
     std::vector<int> step(n_req, 1);
     std::vector<double *> tallies(n_req);
-    Scratch scratch(&ctx->buffers, ctx->stream);
+    Scratch scratch(ctx->buffers, ctx->stream);
+    size_t total = 0;
     if (!ctx->shared_launch) {
         std::vector<int> by_size(n_req);
         for (int r = 0; r < n_req; ++r) by_size[r] = r;
         std::stable_sort(by_size.begin(), by_size.end(), [&](int a, int b) { return ps[a]->nvox < ps[b]->nvox; });
-        size_t total = 0, left = kBatchTallyBudget;
+        size_t left = kBatchTallyBudget;
         for (int k = 0; k < n_req; ++k) {
             const int r = by_size[k];
             step[r] = tallies_within(ps[r]->nvox, n_batches, left / (n_req - k));
@@ -67,15 +68,12 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             total += ps[r]->nvox * step[r];
             left -= ps[r]->nvox * step[r] * sizeof(double);
         }
-        if (total && scratch.buf.ensure(total)) {
-            g_error.clear();
-            step.assign(n_req, 1);
-        }
+        if (total && !scratch.borrow(total)) step.assign(n_req, 1);
     }
-    if (scratch.buf.p) CK(cudaMemsetAsync(scratch.buf.p, 0, scratch.buf.n * sizeof(double), ctx->stream));
+    if (scratch.p) CK(cudaMemsetAsync(scratch.p, 0, total * sizeof(double), ctx->stream));
     size_t taken = 0;
     for (int r = 0; r < n_req; ++r) {
-        tallies[r] = step[r] > 1 ? scratch.buf.p + taken : ps[r]->tally.p;
+        tallies[r] = step[r] > 1 ? scratch.p + taken : ps[r]->tally.p;
         if (step[r] > 1) taken += ps[r]->nvox * step[r];
     }
     std::vector<ctd::FoldDesc> folds(static_cast<size_t>(n_batches) * n_req);
@@ -363,7 +361,7 @@ int admit(ctd_ctx *ctx, bool chains)
         }
         size_t free_b = 0, total_b = 0;
         CK(cudaMemGetInfo(&free_b, &total_b));
-        free_b += ctx->buffers.cached;   // released buffers the context holds for reuse
+        free_b += ctx->buffers.idle();   // what the context holds and an allocation may take back
         const double need = P->tally.p ? 0.0 : 6.0 * 8.0 * static_cast<double>(P->nvox);
         if (static_cast<double>(free_b) < need + ctx->reserve_bytes) break;
         int rc;

@@ -39,14 +39,19 @@ int fail(int code, const char *fmt, ...);
     } while (0)
 
 // Device buffers a context has released and may hand out again: the byte size of
-// each, up to `cap` bytes in all.  A phantom's buffers return here when it is
-// destroyed (after its context's stream is idle), so a phantom of the same size
-// created next takes them without cudaMalloc, and no cudaFree synchronises the
-// device meanwhile.  The context frees what is left when it is destroyed.
+// each, up to `cap` bytes in all, and one block of scratch memory that a call borrows
+// while it runs.  A phantom's buffers return here when it is destroyed (after its
+// context's stream is idle), so a phantom of the same size created next takes them
+// without cudaMalloc, and no cudaFree synchronises the device meanwhile.  The context
+// frees what is left when it is destroyed; what is idle is given back to the device
+// when an allocation finds no memory.
 struct BufferCache {
     std::multimap<size_t, void *> blocks;
     size_t cached = 0;
     size_t cap = size_t(4) << 30;
+    void *scratch = nullptr;
+    size_t scratch_bytes = 0;
+    bool scratch_lent = false;
     void *take(size_t bytes)
     {
         auto it = blocks.find(bytes);
@@ -63,9 +68,51 @@ struct BufferCache {
         cached += bytes;
         return true;
     }
-    ~BufferCache()
+    // bytes that drop() would free
+    size_t idle() const { return cached + (scratch_lent ? 0 : scratch_bytes); }
+    void drop()
     {
         for (auto &b : blocks) cudaFree(b.second);
+        blocks.clear();
+        cached = 0;
+        drop_scratch();
+    }
+    void drop_scratch()
+    {
+        if (scratch_lent || !scratch) return;
+        cudaFree(scratch);
+        scratch = nullptr;
+        scratch_bytes = 0;
+    }
+    // cudaMalloc, once more after giving idle memory back
+    void *allocate(size_t bytes)
+    {
+        void *p = nullptr;
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        if (!idle()) return nullptr;
+        drop();
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
+    }
+    // The scratch block, of at least `bytes` (it only grows); nullptr if it is lent
+    // already or there is no memory.
+    void *borrow(size_t bytes)
+    {
+        if (scratch_lent) return nullptr;
+        if (scratch_bytes < bytes) {
+            drop_scratch();
+            if (!(scratch = allocate(bytes))) return nullptr;
+            scratch_bytes = bytes;
+        }
+        scratch_lent = true;
+        return scratch;
+    }
+    ~BufferCache()
+    {
+        scratch_lent = false;
+        drop();
     }
 };
 
@@ -86,15 +133,14 @@ struct DevBuf {
         if (count <= n && p) return CTD_OK;
         release();
         if (count == 0) count = 1;
-        if (cache && (p = static_cast<T *>(cache->take(count * sizeof(T))))) {
-            n = count;
-            return CTD_OK;
-        }
-        if (cudaMalloc(reinterpret_cast<void **>(&p), count * sizeof(T)) != cudaSuccess) {
+        if (cache) {
+            p = static_cast<T *>(cache->take(count * sizeof(T)));
+            if (!p) p = static_cast<T *>(cache->allocate(count * sizeof(T)));
+        } else if (cudaMalloc(reinterpret_cast<void **>(&p), count * sizeof(T)) != cudaSuccess) {
             cudaGetLastError();
             p = nullptr;
-            return fail(CTD_ENOMEM, "cudaMalloc of %zu bytes failed", count * sizeof(T));
         }
+        if (!p) return fail(CTD_ENOMEM, "cudaMalloc of %zu bytes failed", count * sizeof(T));
         n = count;
         return CTD_OK;
     }
@@ -164,17 +210,21 @@ struct Phantom {
     }
 };
 
-// Device scratch of one call, taken from the context's released buffers and given back
-// when the call ends, then idle (after a failed call the stream is waited for first).
+// The context's scratch block for the length of one call (on stream s, which is waited
+// for if the call fails).
 struct Scratch {
-    DevBuf<double> buf;
+    BufferCache &cache;
     cudaStream_t stream;
-    bool idle = false;
-    Scratch(BufferCache *c, cudaStream_t s) : stream(s) { buf.cache = c; }
+    double *p = nullptr;
+    bool idle = false;   // set once the call has waited for its work
+    Scratch(BufferCache &c, cudaStream_t s) : cache(c), stream(s) {}
     ~Scratch()
     {
-        if (buf.p && !idle) cudaStreamSynchronize(stream);
+        if (!p) return;
+        if (!idle) cudaStreamSynchronize(stream);
+        cache.scratch_lent = false;
     }
+    bool borrow(size_t doubles) { return (p = static_cast<double *>(cache.borrow(doubles * sizeof(double)))) != nullptr; }
 };
 
 struct ServeReq {

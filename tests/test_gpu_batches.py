@@ -106,3 +106,21 @@ def test_histories_across_an_upper_word(ctd, contexts, oracle, a, b):
     ctd.ctd_destroy_phantom(c, h)
     assert whole[1] == parts[1] and whole[1][-1] == int(dev["steps"].sum())
     assert np.allclose(whole[0], parts[0], rtol=1e-12, atol=0)
+
+
+def test_groups_of_batches_of_a_large_grid(ctd, contexts):
+    # 33.6 M voxels: four tallies fit side by side into the scratch memory, so five
+    # batches take two launches and two folds
+    p = I.cbct_water(30_001, 5, seed=13, shape=(256, 256, 512), d=0.1)
+    out = []
+    for c in contexts:
+        dose, sd, st, h = ctd.run_problem(c, p)
+        ctd.ctd_destroy_phantom(c, h)
+        out.append((dose, sd, st))
+    (d0, s0, t0), (d1, s1, t1) = out
+    assert t0["transport_launches"] == 2 and t1["transport_launches"] == 5
+    assert [t0[k] for k in COUNTS] == [t1[k] for k in COUNTS]
+    assert np.allclose(d0, d1, rtol=1e-12, atol=0)
+    assert np.allclose(s0 ** 2, s1 ** 2, rtol=1e-9, atol=1e-12 * float((d0 ** 2).max()))
+    assert t0["avg_rsd"] == pytest.approx(t1["avg_rsd"], rel=1e-9)
+    assert t0["e_deposited_kev"] == pytest.approx(t1["e_deposited_kev"], rel=1e-12)
