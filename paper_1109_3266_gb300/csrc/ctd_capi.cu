@@ -366,7 +366,6 @@ int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t
 ctd::FoldLast last_of(Phantom &P, int nb, bool keep_sums)
 {
     ctd::FoldLast l;
-    l.nb = nb;
     l.inv_nb = 1.0 / nb;
     l.inv_nn = 1.0 / (static_cast<double>(nb) * (nb - 1));
     l.dose = P.dose.p;

@@ -227,12 +227,11 @@ struct FoldBatches {
     int clear;
 };
 
-// The results of a fold that is a run's last: dose and standard error over nb batches
-// (inv_nb = 1/nb, inv_nn = 1/(nb (nb - 1))), and in `partials` (kPartialDoubles) what
+// The results of a fold that is a run's last: dose and standard error over its nb
+// batches (inv_nb = 1/nb, inv_nn = 1/(nb (nb - 1))), and in `partials` (kPartialDoubles) what
 // launch_rsd goes on from.  keep_sums: the batch sums are stored too (more batches may
 // follow).
 struct FoldLast {
-    int nb;
     double inv_nb, inv_nn;
     double *dose, *sd;
     const float *rho;

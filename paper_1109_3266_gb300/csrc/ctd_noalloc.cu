@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kThreads) na_rsd_kernel(const double *__restri
         __longlong_as_double(max_of(reinterpret_cast<const long long *>(scratch + kOffMax), gridDim.x));
     rsd_sums(dose, sd, rho, nvox, dmax, scratch + kOffSums, kMaxStatBlocks);
     if (last_block(reinterpret_cast<unsigned *>(scratch + kOffCells)))
-        rsd_result(scratch + kOffSums, kMaxStatBlocks, gridDim.x, dmax, result);
+        rsd_result<false>(scratch + kOffSums, kMaxStatBlocks, gridDim.x, dmax, nullptr, 0, result);
 }
 
 std::mutex g_mu;

@@ -31,13 +31,14 @@ __device__ __forceinline__ void fold_voxel(double t, size_t v, double *__restric
 }
 
 // Mean over nb batches and its standard error: s^2 = (sum d^2 - nb D^2) / (nb (nb - 1)),
-// with inv_nb = 1/nb and inv_nn = 1/(nb (nb - 1)).
-__device__ __forceinline__ void mean_sd(double s1, double s2, int nb, double inv_nb, double inv_nn, double &D,
-                                        double &sd)
+// nb D^2 as D sum d, with inv_nb = 1/nb and inv_nn = 1/(nb (nb - 1)).  (A comparison of
+// doubles is FP64 work too: the variance's sign and size are read from its bits.)
+__device__ __forceinline__ void mean_sd(double s1, double s2, double inv_nb, double inv_nn, double &D, double &sd)
 {
     D = s1 * inv_nb;
-    const double var = (s2 - nb * D * D) * inv_nn;
-    sd = var > 0.0 ? (var >= 0x1p-1000 ? root(var) : sqrt(var)) : 0.0;
+    const double var = fma(-D, s1, s2) * inv_nn;
+    const int hi = __double2hiint(var);
+    sd = hi >= ((1023 - 1000) << 20) ? root(var) : hi >= 0 ? sqrt(var) : 0.0;
 }
 
 // Fold of a request's batches in one pass, and with kLast the mean, the standard
@@ -46,7 +47,7 @@ __device__ __forceinline__ void mean_sd(double s1, double s2, int nb, double inv
 // binary64 operations a voxel, sum t and sum t^2 (fused), and the weights are applied
 // to the sums: sum d = w sum t, sum d^2 = w^2 sum t^2, for the larger and the smaller
 // batches apart.  kFirst: the sums start here.  Bound by the binary64 pipe (about
-// 2 nb + 20 operations) and by memory (8 bytes a batch and at most 84 once).
+// 2 nb + 15 operations) and by memory (8 bytes a batch and at most 84 once).
 template <bool kFirst, bool kLast>
 __global__ void __launch_bounds__(kThreads) fold_kernel(const FoldBatches f, const double *__restrict__ rinv,
                                                         double *__restrict__ sum_d, double *__restrict__ sum_d2,
@@ -77,13 +78,14 @@ __global__ void __launch_bounds__(kThreads) fold_kernel(const FoldBatches f, con
         const double r = rinv[v];
         if (f.n_first > 0) {
             const double w = f.scale0 * r;
-            e += t1[0];
-            s1 = fma(w, t1[0], s1);
-            s2 = fma(w * w, t2[0], s2);
+            e = kFirst ? t1[0] : e + t1[0];
+            s1 = kFirst ? w * t1[0] : fma(w, t1[0], s1);
+            s2 = kFirst ? (w * w) * t2[0] : fma(w * w, t2[0], s2);
         }
         if (f.n_first < f.nb) {
             const double w = f.scale1 * r;
-            e += t1[1];
+            const bool start = kFirst && f.n_first == 0;
+            e = start ? t1[1] : e + t1[1];
             s1 = fma(w, t1[1], s1);
             s2 = fma(w * w, t2[1], s2);
         }
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(kThreads) fold_kernel(const FoldBatches f, con
         }
         if (kLast) {
             double D, s;
-            mean_sd(s1, s2, last.nb, last.inv_nb, last.inv_nn, D, s);
+            mean_sd(s1, s2, last.inv_nb, last.inv_nn, D, s);
             last.dose[v] = D;
             last.sd[v] = s;
             if (last.rho[v] >= 0.1f) dmax = max_dose(dmax, D);
@@ -122,11 +124,8 @@ __global__ void __launch_bounds__(kThreads) rsd_kernel(const double *__restrict_
     const double dmax = __longlong_as_double(max_of(reinterpret_cast<const long long *>(partials), n_fold));
     double *sums = partials + 2 * kMaxStatBlocks;
     rsd_sums(dose, sd, rho, nvox, dmax, sums, kMaxStatBlocks);
-    if (last_block(reinterpret_cast<unsigned *>(partials + kPartialCells))) {
-        rsd_result(sums, kMaxStatBlocks, gridDim.x, dmax, result);
-        const double e = total_of(partials + kMaxStatBlocks, n_fold);
-        if (threadIdx.x == 0) result[3] = e;
-    }
+    if (last_block(reinterpret_cast<unsigned *>(partials + kPartialCells)))
+        rsd_result<true>(sums, kMaxStatBlocks, gridDim.x, dmax, partials + kMaxStatBlocks, n_fold, result);
 }
 
 // The same fold for several requests at once, one tile of kFoldTile voxels per step.

@@ -45,7 +45,7 @@ __device__ __forceinline__ double root(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    double g = x * y, h = 0.5 * y;
+    double g = x * y, h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));   // y / 2
     const double r = fma(-g, h, 0.5);
     g = fma(g, r, g);
     h = fma(h, r, h);
@@ -215,16 +215,24 @@ __device__ __forceinline__ double total_of(const double *p, int n)
     return x[0];
 }
 
-// result[0..2] = avg RSD, sigma-bar, D_max from n blocks' partial sums
-__device__ __forceinline__ void rsd_result(const double *sums, int stride, int n, double dmax, double *result)
+// result[0..2] = avg RSD, sigma-bar, D_max from n blocks' partial sums, and with extra
+// partials (n_extra of them) result[3] = their sum; the sums are reduced side by side
+template <bool kExtra>
+__device__ __forceinline__ void rsd_result(const double *sums, int stride, int n, double dmax, const double *extra,
+                                           int n_extra, double *result)
 {
-    double s[4];
+    double s[kExtra ? 5 : 4] = {};
+    for (int i = threadIdx.x; i < n; i += kThreads)
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] = total_of(sums + k * stride, n);
+        for (int k = 0; k < 4; ++k) s[k] += __ldcg(sums + k * stride + i);
+    if (kExtra)
+        for (int i = threadIdx.x; i < n_extra; i += kThreads) s[kExtra ? 4 : 0] += __ldcg(extra + i);
+    block_sum<kExtra ? 5 : 4>(s);
     if (threadIdx.x == 0) {
         result[0] = s[1] > 0.0 ? s[0] / s[1] : 0.0;
         result[1] = (s[3] > 0.0 && dmax > 0.0) ? s[2] / (s[3] * dmax) : 0.0;
         result[2] = dmax;
+        if (kExtra) result[3] = s[kExtra ? 4 : 0];
     }
 }
 
