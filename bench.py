@@ -56,13 +56,14 @@ FLUSH_BYTES = 256 * 1024 * 1024
 # (smsp__thread_inst_executed / histories) and DRAM bytes per launch
 # (dram__bytes_read + dram__bytes_write); they are not measured in this run.
 KERNEL_PROFILE = {
-    "cbct_water": {"lane_inst_per_history": 2088.0, "dram_bytes_per_launch": 4.345e9, "histories_per_launch": 1e8,
-                   "capture": "ncu --set full --clock-control none of one transport_kernel<256,4,0,0> launch of 1e8 "
-                              "CBCT-water histories (packed-voxel kernel): 8.688e9 warp instructions x 24.03 lanes; "
-                              "DRAM 1.91 + 2.43 GB"},
-    "head": {"lane_inst_per_history": 2450.0, "dram_bytes_per_launch": 4.465e9, "histories_per_launch": 2e8,
-             "capture": "ncu --set full --clock-control none of one transport_kernel<256,4,0,0> launch of 2e8 head "
-                        "histories (packed-voxel kernel): 2.656e10 warp instructions x 18.45 lanes; DRAM 2.53 + 1.94 GB"},
+    "cbct_water": {"lane_inst_per_history": 1863.0, "dram_bytes_per_launch": 1.540e9, "histories_per_launch": 4e7,
+                   "capture": "ncu --set full --clock-control none of one transport_kernel<384,3,0> launch of 4e7 "
+                              "CBCT-water histories in 2 batches (straight-line kernel): 2.772e9 warp instructions x "
+                              "26.88 lanes; DRAM 0.70 + 0.85 GB"},
+    "head": {"lane_inst_per_history": 2261.0, "dram_bytes_per_launch": 0.765e9, "histories_per_launch": 4e7,
+             "capture": "ncu --set full --clock-control none of one transport_kernel<384,3,0> launch of 4e7 head "
+                        "histories in 2 batches (straight-line kernel): 4.287e9 warp instructions x 21.10 lanes; "
+                        "DRAM 0.46 + 0.31 GB"},
 }
 
 
@@ -450,7 +451,8 @@ def leg_head(ctd, args, stream, flush, peaks, peak_kind, clk):
     if not args.no_cpu_baseline:
         _, _, _, ranges, edep, c = oracle_sample(p, 3.0, cpu_cores(), keep=True)
         out["error_vs_fp64_oracle"] = error_vs_oracle(ctd, ctx, h, p, ranges, edep, c)
-    out["gpu_launches"] = run["launches"] + 17 * args.head_steps
+    # a fold follows each transport launch, the precision measures each run
+    out["gpu_launches"] = 2 * run["launches"] + args.head_steps
     ctd.ctd_destroy_phantom(ctx, h)
     ctd.ctd_destroy(ctx)
     return out
@@ -686,7 +688,8 @@ def run_ours(args):
     probes = None if args.no_probe else memory_probes(ctd, ctx, nvox)
     prof = KERNEL_PROFILE.get(p.name) if args.compton == "kn" and args.rayleigh == "gauss" else None
     line["roofline"] = roofline(p, run, peaks, peak_kind, probes, prof)
-    line["gpu_launches"] = run["launches"] + 17 * args.steps
+    # a fold follows each transport launch, the precision measures each run
+    line["gpu_launches"] = 2 * run["launches"] + args.steps
     if not args.no_cpu_baseline:
         threads = cpu_cores()
         r, n, dt, ranges, edep, c = oracle_sample(p, args.ref_seconds, threads, keep=True)

@@ -45,36 +45,50 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     if ((rc = ctx->u_work.ensure(static_cast<size_t>(n_batches) * n_req))) return rc;
     // descriptors for every batch of every request, the history and tile offsets
     std::vector<ctd::RequestDesc> descs(static_cast<size_t>(n_batches) * n_req);
-    // Request chains: batches of a request share launches as in a plain run, each with a
-    // tally in the call's scratch memory, cleared before the graph runs.  The requests
-    // share kBatchTallyBudget, those with the smallest grids first, each up to an equal
-    // share of what is left; one that gets room for a single tally (or every one, without
-    // room for the scratch) uses its phantom's.  16 requests of 64^3 to 128^3 voxels and
-    // 1e6 to 1e7 histories: 7.7 ms on the GPU with every batch in one launch, 12.8 ms with
-    // the larger grids' batches in launches of their own, 9.7 ms one ctd_run after another.
-    std::vector<int> step(n_req, 1);
+    // Request chains are issued largest first (so that the last to finish are short ones:
+    // longest processing time first), the k-th on stream k mod n_lanes.  Batches of a
+    // request share launches as in a plain run, each with a tally in the call's scratch
+    // memory; chains that share a stream share its part of that, which a fold leaves
+    // cleared for the next.  Fewer streams are used where the largest grids' tallies would
+    // not fit kBatchTallyBudget otherwise (two at least): 64 requests of 64^3 to 256^3
+    // voxels, 1.28e10 histories, took 1196 ms on 64 streams with most batches in launches
+    // of their own, 1056 ms on three with all of a request's in one, 1083 ms one ctd_run
+    // after another; 16 requests of 64^3 to 128^3 voxels 12.8, 7.7 and 9.7 ms.
+    std::vector<int> order(n_req), step(n_req, 1);
+    for (int r = 0; r < n_req; ++r) order[r] = r;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n_histories[a] > n_histories[b]; });
     std::vector<double *> tallies(n_req);
+    for (int r = 0; r < n_req; ++r) tallies[r] = ps[r]->tally.p;
+    int n_lanes = std::min(n_req, ctx->batch_lanes);
     Scratch scratch(ctx->buffers, ctx->stream);
-    size_t total = 0;
     if (!ctx->shared_launch) {
-        std::vector<int> by_size(n_req);
-        for (int r = 0; r < n_req; ++r) by_size[r] = r;
-        std::stable_sort(by_size.begin(), by_size.end(), [&](int a, int b) { return ps[a]->nvox < ps[b]->nvox; });
-        size_t left = kBatchTallyBudget;
-        for (int k = 0; k < n_req; ++k) {
-            const int r = by_size[k];
-            step[r] = tallies_within(ps[r]->nvox, n_batches, left / (n_req - k));
-            if (step[r] == 1) continue;
-            total += ps[r]->nvox * step[r];
-            left -= ps[r]->nvox * step[r] * sizeof(double);
+        // voxels of scratch each of `lanes` streams needs for every batch of its requests,
+        // within an equal share of the budget
+        auto parts = [&](int lanes) {
+            std::vector<size_t> need(lanes, 0);
+            for (int k = 0; k < n_req; ++k) {
+                const int r = order[k];
+                step[r] = tallies_within(ps[r]->nvox, n_batches, kBatchTallyBudget / lanes);
+                if (step[r] > 1) need[k % lanes] = std::max(need[k % lanes], ps[r]->nvox * step[r]);
+            }
+            return need;
+        };
+        auto whole = [&] { return std::all_of(step.begin(), step.end(), [&](int g) { return g == n_batches; }); };
+        std::vector<size_t> need = parts(n_lanes);
+        while (!whole() && n_lanes > 2) need = parts(--n_lanes);
+        size_t total = 0;
+        for (size_t v : need) total += v;
+        if (total && !scratch.borrow(total)) {
+            step.assign(n_req, 1);
+            n_lanes = std::min(n_req, ctx->batch_lanes);
         }
-        if (total && !scratch.borrow(total)) step.assign(n_req, 1);
-    }
-    if (scratch.p) CK(cudaMemsetAsync(scratch.p, 0, total * sizeof(double), ctx->stream));
-    size_t taken = 0;
-    for (int r = 0; r < n_req; ++r) {
-        tallies[r] = step[r] > 1 ? scratch.p + taken : ps[r]->tally.p;
-        if (step[r] > 1) taken += ps[r]->nvox * step[r];
+        if (scratch.p) {
+            CK(cudaMemsetAsync(scratch.p, 0, total * sizeof(double), ctx->stream));
+            std::vector<size_t> first(n_lanes, 0);
+            for (int l = 1; l < n_lanes; ++l) first[l] = first[l - 1] + need[l - 1];
+            for (int k = 0; k < n_req; ++k)
+                if (step[order[k]] > 1) tallies[order[k]] = scratch.p + first[k % n_lanes];
+        }
     }
     std::vector<ctd::FoldDesc> folds(static_cast<size_t>(n_batches) * n_req);
     std::vector<uint64_t> tiles(n_req + 1, 0);
@@ -137,18 +151,12 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             fill_shared(*ps[r], sh);
             put(&sh, sizeof(sh));
         }
-        const int n_lanes = std::min(n_req, ctx->batch_lanes);
         if ((rc = ensure_lanes(ctx, n_lanes))) return rc;
         if (!event_at(ctx, 0) || !event_at(ctx, 1)) return fail(CTD_ECUDA, "cudaEventCreate failed");
-        // chains are issued largest first, so that the last to finish are short ones
-        // (longest processing time first: the smaller requests fill the tail)
-        std::vector<int> order(n_req);
-        for (int r = 0; r < n_req; ++r) order[r] = r;
-        std::stable_sort(order.begin(), order.end(),
-                         [&](int a, int b) { return n_histories[a] > n_histories[b]; });
         put(order.data(), order.size() * sizeof(int));
         put(step.data(), step.size() * sizeof(int));
-        body = [&, order, n_lanes](cudaStream_t cs) {
+        put(&n_lanes, sizeof(n_lanes));
+        body = [&](cudaStream_t cs) {
             if (cudaMemsetAsync(ctx->u_work.p, 0, static_cast<size_t>(n_batches) * n_req * sizeof(unsigned long long),
                                 cs) != cudaSuccess ||
                 cudaEventRecordWithFlags(ctx->events[0], cs, cudaEventRecordExternal) != cudaSuccess)
@@ -157,16 +165,15 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             for (int k = 0; k < n_req && e == CTD_OK; ++k) {
                 const int r = order[k];
                 Phantom &P = *ps[r];
-                // the k-th largest request on lane k (mod the lanes)
                 const cudaStream_t ls = ctx->lanes[k % n_lanes];
                 const ctd::FoldLast last = last_of(P, n_batches, false);
                 for (int b = 0; b < n_batches && e == CTD_OK; b += step[r]) {
                     const size_t d = static_cast<size_t>(b) * n_req + r;
                     const int g = std::min(step[r], n_batches - b);
-                    // (a fold clears the tallies for the batches that follow it)
+                    // (a fold clears the tallies for what follows on the stream)
                     e = launch_one(ctx, P, descs[d], ls);
                     if (e == CTD_OK)
-                        e = ctd::launch_fold(fold_of(P, n_histories[r], n_batches, b, g, tallies[r], b + g < n_batches), P.rinv.p,
+                        e = ctd::launch_fold(fold_of(P, n_histories[r], n_batches, b, g, tallies[r], true), P.rinv.p,
                                              P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, b == 0,
                                              b + g == n_batches ? &last : nullptr, ls);
                 }

@@ -251,7 +251,7 @@ struct ServeReq {
 
 // device memory a plain run may take, while it runs, for the tallies of batches that
 // share a launch, and a batched call for all its requests'
-constexpr size_t kTallyBudget = size_t(1) << 30, kBatchTallyBudget = size_t(2) << 30;
+constexpr size_t kTallyBudget = size_t(1) << 30, kBatchTallyBudget = size_t(4) << 30;
 constexpr int kMaxLanes = 64;     // streams for request chains
 constexpr uint64_t kMaxTrace = 1ull << 26;   // histories of one trace call (16 B of device memory each)
 

@@ -49,9 +49,13 @@ def test_shared_launch_equals_launch_per_batch(ctd, contexts, n, nb):
     assert np.allclose(s0 ** 2, s1 ** 2, rtol=1e-9, atol=1e-12 * float((d0 ** 2).max()))
 
 
-def test_batched_chains_share_launches_like_plain_runs(ctd, contexts):
-    ps = [I.head(10_007, 6, seed=3, shape=(24, 20, 16), d=1.0), I.cbct_water(200_001, 6, seed=4, shape=(32, 30, 8), d=0.8)]
-    c = contexts[0]
+@pytest.mark.parametrize("lanes", [0, 1, 2])
+def test_batched_chains_share_launches_like_plain_runs(ctd, contexts, lanes):
+    # (with fewer streams than requests, chains share scratch tallies one after another)
+    ps = [I.head(10_007, 6, seed=3, shape=(24, 20, 16), d=1.0), I.cbct_water(200_001, 6, seed=4, shape=(32, 30, 8), d=0.8),
+          I.head(60_000, 6, seed=5, shape=(40, 38, 30), d=0.5), I.cbct_water(7_000, 6, seed=6, shape=(16, 16, 16), d=1.0),
+          I.head(33_333, 6, seed=7, shape=(20, 44, 18), d=0.8)]
+    c = ctd.ctd_create(device=0, batch_lanes=lanes)
     hs = [ctd.load_problem(c, p) for p in ps]
     for _ in range(2):   # recorded, then replayed
         ctd.ctd_run_batch(c, hs, [p.n_hist for p in ps], [p.seed for p in ps], 6)
@@ -60,7 +64,7 @@ def test_batched_chains_share_launches_like_plain_runs(ctd, contexts):
         d1, s1, t1, _ = ctd.run_problem(contexts[1], p)
         assert [st[k] for k in COUNTS] == [t1[k] for k in COUNTS]
         assert np.allclose(dose, d1, rtol=1e-12, atol=0)
-        ctd.ctd_destroy_phantom(c, h)
+    ctd.ctd_destroy(c)
 
 
 @pytest.mark.parametrize("n_mat,e_max", [(1, 150), (16, 150), (16, 400), (16, 780)])
