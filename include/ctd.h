@@ -50,8 +50,9 @@ typedef struct {
     int blocks_per_sm;        /* transport grid = SMs x blocks_per_sm (default 4)     */
     int threads_per_block;    /* multiple of 32, <= 256 (default 256; single requests at
                                  4 blocks of 256 per SM run as 3 blocks of 384)       */
-    int chunk;                /* histories a warp claims at a time (default 256; at most 32
-                                 of a launch's last ones, some 256 per warp)          */
+    int chunk;                /* histories a warp claims at a time, at most (default 256;
+                                 fewer in a launch alone with fewer than 16 such per warp,
+                                 at most 32 of a launch's last ones, some 256 per warp) */
     int flight_cap;           /* Woodcock flights a lane takes in a row, stopping early at a
                                  real interaction, before its warp moves on (default 4) */
     int multi_blocks_per_sm;  /* grid of multi-request launches (batched, served; default 3) */

@@ -357,10 +357,9 @@ int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t
     std::memset(&L, 0, sizeof(L));
     fill_shared(P, L.sh);
     L.one = q;
-    L.chunk = ctx->chunk;
     L.flight_cap = ctx->flight_cap;
     const LaunchShape shape = launch_shape(ctx, L.sh, q.mode, false);
-    return launch_single(L, shape, s);
+    return launch_single(ctx, L, shape, s);
 }
 
 ctd::FoldLast last_of(Phantom &P, int nb, bool keep_sums)
@@ -405,11 +404,22 @@ LaunchShape launch_shape(const ctd_ctx *ctx, const ctd::SharedTables &sh, int mo
     return {ctx->num_sms * ctx->blocks_per_sm, ctx->threads, ctx->threads * ctx->blocks_per_sm};
 }
 
-// Claims: runs of `chunk` histories until what is left is some 256 per warp, then of
-// 32, one round of source photons.  1e6 histories (a 51x51x32 head, 183 per warp) took
-// 0.43 ms while half of them went in claims of 256, 0.24 in claims of 32; for 1e5 claims
-// of 18, so that every warp has one, took 0.080 ms, claims of 32 0.057.
-static void set_claims(ctd::RequestDesc &q, uint64_t h0, uint64_t h1, int chunk, int warps)
+// Claims: `chunk` histories each (for a launch that has the GPU to itself at most a
+// sixteenth of a warp's share of it) until what is left is some 256 per warp, then 32,
+// one round of source photons.  1e6 histories (a 51x51x32 head, 183 per warp) took 0.43 ms
+// while half of them went in claims of 256, 0.23 in claims of 32; for 1e5 claims of 18, so
+// that every warp has one, took 0.080 ms, claims of 32 0.057.
+// With claims of 256 in every launch of more than 256 per warp the first round alone was
+// 1.4e6 histories, and a warp that met a costly run of them (a batch's histories go from
+// low energies to high) ended last: 1.5e6 histories took 0.454 ms, now 0.285; 4e6 0.701 ->
+// 0.567 (head), 0.384 -> 0.362 (water); 1e7 1.350 -> 1.286; from some 2e7 nothing changes,
+// where claims of 64 throughout would cost 2 to 5 %.  An eighth of a share lost 4 to 8 % at
+// 4e6 to 1e7 on heads, a thirtieth 2 to 3 % on water.  Beside other launches (streams of
+// chains, overlapped batches, requests of one launch) the tails are filled anyway and
+// smaller claims only cost: eight served requests of 4e6 histories a batch 108 -> 113 ms,
+// overlapped batches of 2.5e6 water histories 0.97 -> 1.03.
+constexpr int kClaimsPerWarp = 16;
+static void set_claims(ctd::RequestDesc &q, uint64_t h0, uint64_t h1, int chunk, int warps, bool alone)
 {
     const uint64_t larger = q.rem * (q.n_lo + 1);   // histories in the larger batches
     q.b0 = static_cast<int>(h0 < larger ? h0 / (q.n_lo + 1) : q.rem + (h0 - larger) / q.n_lo);
@@ -417,22 +427,25 @@ static void set_claims(ctd::RequestDesc &q, uint64_t h0, uint64_t h1, int chunk,
     q.h_end = h1;
     const uint64_t tail = 256 * static_cast<uint64_t>(std::max(warps, 1));
     q.h_big = h1 - h0 > tail ? h1 - tail : h0;
+    const uint64_t share = (h1 - h0) / (kClaimsPerWarp * static_cast<uint64_t>(std::max(warps, 1)));
+    q.big = alone ? static_cast<int>(std::min<uint64_t>((share / 32 + 1) * 32, chunk)) : chunk;
     q.small = std::min(32, chunk);
     q.h_hi = static_cast<uint32_t>(h0 >> 32);
     q.k0 = q.rk[0] ^ q.h_hi;
 }
 
 void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1, double *tally, uint32_t stride,
-               int chunk, int warps)
+               int chunk, int warps, bool alone)
 {
     q.n_lo = n / nb;
     q.rem = n % nb;
     q.tally = tally;
     q.tally_stride = stride;
-    set_claims(q, h0, h1, chunk, warps);
+    set_claims(q, h0, h1, chunk, warps, alone);
 }
 
-int launch_single(ctd::LaunchParams &L, const LaunchShape &shape, cudaStream_t s, const ctd::L2Window *win)
+int launch_single(const ctd_ctx *ctx, ctd::LaunchParams &L, const LaunchShape &shape, cudaStream_t s,
+                  const ctd::L2Window *win)
 {
     ctd::RequestDesc &q = L.one;
     const uint64_t end = q.h_end;
@@ -442,7 +455,7 @@ int launch_single(ctd::LaunchParams &L, const LaunchShape &shape, cudaStream_t s
         const uint64_t last = h | 0xffffffffull;   // the last history with this upper word
         if (h != q.h_begin || last < end - 1) {
             if (h != q.h_begin && cudaMemsetAsync(q.work, 0, sizeof(unsigned long long), s) != cudaSuccess) return CTD_ECUDA;
-            set_claims(q, h, last < end - 1 ? last + 1 : end, L.chunk, warps);
+            set_claims(q, h, last < end - 1 ? last + 1 : end, ctx->chunk, warps, true);
             q.tally = tally + static_cast<size_t>(q.b0 - b0) * q.tally_stride;
         }
         const int rc = ctd::launch_transport(L, shape.grid, shape.block, shape.threads_per_sm, s, win);
@@ -479,10 +492,9 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb,
     L.trace_n = trace_n;
     fill_shared(P, L.sh);
     const LaunchShape shape = launch_shape(ctx, L.sh, q.mode, trace != nullptr);
-    set_range(q, n, nb, h0, h1, tally, stride, ctx->chunk, shape.grid * (shape.block / 32));
+    set_range(q, n, nb, h0, h1, tally, stride, ctx->chunk, shape.grid * (shape.block / 32), !ctx->plain_overlap);
     q.work = work;
     L.one = q;
-    L.chunk = ctx->chunk;
     L.flight_cap = ctx->flight_cap;
     if (clear_work) CK(cudaMemsetAsync(work, 0, sizeof(unsigned long long), s));
     cudaEvent_t e0 = event_at(ctx, 2 * ev_index), e1 = event_at(ctx, 2 * ev_index + 1);
@@ -502,7 +514,7 @@ int transport(ctd_ctx *ctx, Phantom &P, ctd::RequestDesc &q, uint64_t n, int nb,
         }
         win.hit_ratio = static_cast<float>(std::min(1.0, static_cast<double>(ctx->l2_setaside) / win.bytes));
     }
-    CKS(launch_single(L, shape, s, ctx->l2_persist ? &win : nullptr));
+    CKS(launch_single(ctx, L, shape, s, ctx->l2_persist ? &win : nullptr));
     CK(cudaEventRecord(e1, s));
     return CTD_OK;
 }

@@ -118,7 +118,8 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             const LaunchShape one = launch_shape(ctx, sh, q.mode, false);
             set_range(q, n, n_batches, h0, h1, tallies[r], ctx->shared_launch ? 0 : static_cast<uint32_t>(nv), ctx->chunk,
                       ctx->shared_launch ? ctx->num_sms * ctx->multi_blocks_per_sm * ctx->threads / 32
-                                         : one.grid * (one.block / 32));
+                                         : one.grid * (one.block / 32),
+                      !ctx->shared_launch && n_lanes == 1);
             q.work = ctx->u_work.p + static_cast<size_t>(b) * n_req + r;
             ctd::FoldDesc &f = folds[static_cast<size_t>(b) * n_req + r];
             f.tally = P.tally.p;
@@ -209,7 +210,6 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             L.any_fluence |= ps[r]->fl_nu > 0;
             L.sh.wide |= sh.wide;
         }
-        L.chunk = ctx->chunk;
         L.flight_cap = ctx->flight_cap;
         put(&L, sizeof(L));
         const int mgrid = ctx->num_sms * ctx->multi_blocks_per_sm;
@@ -469,7 +469,8 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
         const uint64_t first = static_cast<uint64_t>(R.batches + j) * B;
         const uint64_t h0 = j == 0 ? first + lo : first, h1 = j == 0 ? first + hi : first + B;
         if (h0 < h1) {
-            set_range(q, B * nb, nb, h0, h1, P.tally.p, 0, ctx->chunk, warps);
+            set_range(q, B * nb, nb, h0, h1, P.tally.p, 0, ctx->chunk, warps,
+                      ctx->active.size() == 1);
             CK(cudaMemsetAsync(q.work, 0, sizeof(unsigned long long), s));
             CKS(launch_one(ctx, P, q, s));
             hist += static_cast<double>(h1 - h0);
@@ -688,7 +689,7 @@ int serve_round(ctd_ctx *ctx)
         q.work = ctx->u_work.p + i;
         // batch R.batches of a problem of R.batches + 1 batches of exactly B histories
         set_range(q, B * (R.batches + 1), R.batches + 1, B * R.batches, B * (R.batches + 1), P.tally.p, 0, ctx->chunk,
-                  ctx->num_sms * ctx->multi_blocks_per_sm * ctx->threads / 32);
+                  ctx->num_sms * ctx->multi_blocks_per_sm * ctx->threads / 32, false);
         tiles[i + 1] = tiles[i] + (P.nvox + ctd::kFoldTile - 1) / ctd::kFoldTile;
         ctd::FoldDesc &f = folds[i];
         f.tally = P.tally.p;
@@ -728,7 +729,6 @@ int serve_round(ctd_ctx *ctx)
         L.any_fluence |= ps[i]->fl_nu > 0;
         L.sh.wide |= sh.wide;
     }
-    L.chunk = ctx->chunk;
     L.flight_cap = ctx->flight_cap;
     const int mgrid = ctx->num_sms * ctx->multi_blocks_per_sm;
     if ((rc = ctd::launch_transport(L, mgrid, ctx->threads, ctx->threads * ctx->multi_blocks_per_sm, ctx->stream)) ||

@@ -116,13 +116,12 @@ struct alignas(16) RequestDesc {
     // consecutive histories, the first `rem` of n_lo + 1 and the others of n_lo: batch b
     // starts at b n_lo + min(b, rem).  Deposits of batch b go to tally + (b - b0) tally_stride.
     uint64_t h_begin, h_end;
-    uint64_t h_big;              // claims starting before it take P.chunk histories, later ones `small`
+    uint64_t h_big;              // after a claim ending before it a warp takes `big` histories, then `small`
     uint64_t n_lo, rem;
     int b0;                      // batch of h_begin
     uint32_t tally_stride;       // voxels, or 0: every batch into one grid
-    int small;
+    int big, small;
     uint32_t h_hi, k0;           // single-request launches: upper word of every history's index, and ^ rk[0]
-    int pad_;
     int n_mat;
     int nbins;
     int nx, ny, nz;
@@ -194,7 +193,6 @@ struct LaunchParams {
     RequestDesc one;             // the request of a single-request launch
     const RequestDesc *reqs;     // [n_req] (multi-request launches; n_req == 0: single)
     int n_req;
-    int chunk;                   // histories a warp claims at a time
     int flight_cap;              // Woodcock flights a lane takes before yielding to the warp
     int any_fluence;             // multi-request launches: some request has a fluence map
     // per-history records of a trace launch (single request; nullptr otherwise):

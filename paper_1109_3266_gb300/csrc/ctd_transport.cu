@@ -492,7 +492,7 @@ constexpr size_t kWarpBytes = kQueueBytes + sizeof(WarpPool) + 32 * sizeof(LaneS
 static_assert(kWarpBytes % 16 == 0, "a warp's shared-memory area must keep 16-byte alignment");
 
 // All histories [q.h_begin, q.h_end) of one request, claimed by warps from q.work in
-// runs of P.chunk, near the end of q.small.  A claim's photons carry their batch's
+// runs of q.big, near the end of q.small.  A claim's photons carry their batch's
 // tally with them, so a warp goes from one batch to the next without draining.
 // Returns when the warp has no photon left.
 //
@@ -533,7 +533,7 @@ __device__ __forceinline__ void run_request(const LaunchParams &P, const Request
                 uint64_t end = Q.pool->end, first = Q.pool->first;
                 int batch = Q.pool->batch;
                 if (next >= end) {
-                    const unsigned size = end < q.h_big ? P.chunk : q.small;
+                    const unsigned size = end < q.h_big ? q.big : q.small;
                     unsigned long long base = 0;
                     if (lane == 0) base = atomicAdd(q.work, static_cast<unsigned long long>(size));
                     base = __shfl_sync(kFull, base, 0);

@@ -49,6 +49,22 @@ def test_shared_launch_equals_launch_per_batch(ctd, contexts, n, nb):
     assert np.allclose(s0 ** 2, s1 ** 2, rtol=1e-9, atol=1e-12 * float((d0 ** 2).max()))
 
 
+@pytest.mark.parametrize("n,nb,chunk", [(1_500_001, 4, 0), (2_801_665, 3, 0), (2_801_663, 3, 0), (9_000_011, 6, 0),
+                                        (1_500_001, 4, 40), (5_000_000, 2, 1000)])
+def test_claims_of_a_share_cover_every_history_once(ctd, contexts, n, nb, chunk):
+    # claims of 32 to 256 histories by the launch's size (5472 warps: 32 and 64 meet at
+    # 2801664), at most the option's; a launch per batch claims by each batch's size
+    p = I.head(n, nb, seed=13, shape=(24, 22, 16), d=1.0)
+    c = ctd.ctd_create(device=0, chunk=chunk)
+    d0, s0, t0, h0 = ctd.run_problem(c, p)
+    d1, s1, t1, h1 = ctd.run_problem(contexts[1], p)
+    ctd.ctd_destroy_phantom(contexts[1], h1)
+    ctd.ctd_destroy(c)
+    assert [t0[k] for k in COUNTS] == [t1[k] for k in COUNTS]
+    assert t0["e_emitted_kev"] == t1["e_emitted_kev"] and t0["e_escaped_kev"] == t1["e_escaped_kev"]
+    assert np.allclose(d0, d1, rtol=1e-12, atol=0)
+
+
 @pytest.mark.parametrize("lanes", [0, 1, 2])
 def test_batched_chains_share_launches_like_plain_runs(ctd, contexts, lanes):
     # (with fewer streams than requests, chains share scratch tallies one after another)
