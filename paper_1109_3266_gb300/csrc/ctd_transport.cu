@@ -501,7 +501,8 @@ static_assert(kWarpBytes % 16 == 0, "a warp's shared-memory area must keep 16-by
 // beside warps with none, which is nearly all of a small batch.  Transport of 1e5
 // histories in 10 batches (32^3 water): 0.69 ms in 10 launches -> 0.071 in one; 1e6 in 7
 // (51x51x32 head) 2.83 -> 0.43; 1e7 in 10 (48x48x40 head, helix) 4.31 -> 1.47; 2e8 in 2
-// (CBCT water) 15.29 -> 15.00.
+// (CBCT water) 15.29 -> 15.00.  (With later steps and smaller claims 0.055, 0.23, 1.29 and
+// 13.97.)
 template <bool kMulti, bool kFluence, bool kWide, bool kAnyMode, bool kTrace>
 __device__ __forceinline__ void run_request(const LaunchParams &P, const RequestDesc &q, const float2 *s_tab,
                                             const float *s_mm, const Queue &Q, int lane, LaneCounts &cnt)
