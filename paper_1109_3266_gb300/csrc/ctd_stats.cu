@@ -47,7 +47,8 @@ __device__ __forceinline__ void mean_sd(double s1, double s2, double inv_nb, dou
 // binary64 operations a voxel, sum t and sum t^2 (fused), and the weights are applied
 // to the sums: sum d = w sum t, sum d^2 = w^2 sum t^2, for the larger and the smaller
 // batches apart.  kFirst: the sums start here.  Bound by the binary64 pipe (about
-// 2 nb + 15 operations) and by memory (8 bytes a batch and at most 84 once).
+// 2 nb + 15 operations) and by memory (8 bytes a batch and at most 84 once): 8.4 M voxels
+// and ten batches 0.68 ms, where a fold per batch and a kernel for the mean took 1.49.
 template <bool kFirst, bool kLast>
 __global__ void __launch_bounds__(kThreads) fold_kernel(const FoldBatches f, const double *__restrict__ rinv,
                                                         double *__restrict__ sum_d, double *__restrict__ sum_d2,
