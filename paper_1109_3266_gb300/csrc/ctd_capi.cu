@@ -349,16 +349,14 @@ int ensure_plain_aux(ctd_ctx *ctx, Phantom &P)
     return P.tally2.ensure(P.nvox);
 }
 
-// One single-request launch of q (its tables from P) on stream s, at the
-// context's launch shape.
-int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t s)
+// One single-request launch of q (its tables from P) on stream s.
+int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, const LaunchShape &shape, cudaStream_t s)
 {
     ctd::LaunchParams L;
     std::memset(&L, 0, sizeof(L));
     fill_shared(P, L.sh);
     L.one = q;
     L.flight_cap = ctx->flight_cap;
-    const LaunchShape shape = launch_shape(ctx, L.sh, q.mode, false);
     return launch_single(ctx, L, shape, s);
 }
 

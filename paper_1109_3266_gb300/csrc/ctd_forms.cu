@@ -90,6 +90,26 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
                 if (step[order[k]] > 1) tallies[order[k]] = scratch.p + first[k % n_lanes];
         }
     }
+    // A chain's transport takes a third of the blocks per SM while the chains issued after
+    // it hold at least twice its histories: three chains then share every SM, and one's
+    // tail, folds and measures lie under the others' transport, where launches that each
+    // fill the GPU follow one another with only their tails overlapped.  The last ones and a
+    // dominant one take all blocks, since nothing would fill the rest.  On the GPU, 16
+    // requests of 1e6 to 1e7 histories 6.9 -> 6.0 ms, 64 of 1e5 to 1e6 6.3 -> 4.3, 64 of 1e4
+    // to 1e5 1.20 -> 0.96, 16 of 5e6 9.25 -> 8.5; 24 of 1e7 to 3e8 175 either way.  Two
+    // thirds of the blocks gain half of that.  With three or four streams the large ones
+    // lost 3 %, so six at least.
+    std::vector<LaunchShape> shapes(n_req);
+    uint64_t later = 0;   // histories of the chains issued after this one
+    for (int k = n_req - 1; k >= 0; --k) {
+        const int r = order[k];
+        ctd::SharedTables sh{};
+        fill_shared(*ps[r], sh);
+        LaunchShape &one = shapes[r] = launch_shape(ctx, sh, ps[r]->phys.mode, false);
+        if (!ctx->shared_launch && n_lanes >= 6 && later / 2 >= n_histories[r])
+            one.grid = ctx->num_sms * std::max(one.grid / ctx->num_sms / 3, 1);
+        later += n_histories[r];
+    }
     std::vector<ctd::FoldDesc> folds(static_cast<size_t>(n_batches) * n_req);
     std::vector<uint64_t> tiles(n_req + 1, 0);
     for (int r = 0; r < n_req; ++r)
@@ -113,12 +133,9 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
             const uint64_t h0 = batch_start(n, n_batches, b), h1 = batch_start(n, n_batches, b + k);
             ctd::RequestDesc &q = descs[static_cast<size_t>(b) * n_req + r];
             fill_request(P, seeds[r], q);
-            ctd::SharedTables sh{};
-            fill_shared(P, sh);
-            const LaunchShape one = launch_shape(ctx, sh, q.mode, false);
             set_range(q, n, n_batches, h0, h1, tallies[r], ctx->shared_launch ? 0 : static_cast<uint32_t>(nv), ctx->chunk,
                       ctx->shared_launch ? ctx->num_sms * ctx->multi_blocks_per_sm * ctx->threads / 32
-                                         : one.grid * (one.block / 32),
+                                         : shapes[r].grid * (shapes[r].block / 32),
                       !ctx->shared_launch && n_lanes == 1);
             q.work = ctx->u_work.p + static_cast<size_t>(b) * n_req + r;
             ctd::FoldDesc &f = folds[static_cast<size_t>(b) * n_req + r];
@@ -156,6 +173,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
         if (!event_at(ctx, 0) || !event_at(ctx, 1)) return fail(CTD_ECUDA, "cudaEventCreate failed");
         put(order.data(), order.size() * sizeof(int));
         put(step.data(), step.size() * sizeof(int));
+        put(shapes.data(), shapes.size() * sizeof(LaunchShape));
         put(&n_lanes, sizeof(n_lanes));
         body = [&](cudaStream_t cs) {
             if (cudaMemsetAsync(ctx->u_work.p, 0, static_cast<size_t>(n_batches) * n_req * sizeof(unsigned long long),
@@ -172,7 +190,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
                     const size_t d = static_cast<size_t>(b) * n_req + r;
                     const int g = std::min(step[r], n_batches - b);
                     // (a fold clears the tallies for what follows on the stream)
-                    e = launch_one(ctx, P, descs[d], ls);
+                    e = launch_one(ctx, P, descs[d], shapes[r], ls);
                     if (e == CTD_OK)
                         e = ctd::launch_fold(fold_of(P, n_histories[r], n_batches, b, g, tallies[r], true), P.rinv.p,
                                              P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, b == 0,
@@ -472,7 +490,7 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
             set_range(q, B * nb, nb, h0, h1, P.tally.p, 0, ctx->chunk, warps,
                       ctx->active.size() == 1);
             CK(cudaMemsetAsync(q.work, 0, sizeof(unsigned long long), s));
-            CKS(launch_one(ctx, P, q, s));
+            CKS(launch_one(ctx, P, q, shape, s));
             hist += static_cast<double>(h1 - h0);
         }
         if (j < n)

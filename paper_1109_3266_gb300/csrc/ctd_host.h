@@ -354,8 +354,6 @@ cudaEvent_t event_at(ctd_ctx *ctx, size_t i);
 int ensure_lanes(ctd_ctx *ctx, int n);
 int fork_lanes(ctd_ctx *ctx, cudaStream_t origin, int n);
 int join_lanes(ctd_ctx *ctx, cudaStream_t origin, int n);
-// one single-request launch of q on stream s at the context's launch shape
-int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, cudaStream_t s);
 // the last fold's outputs for a run of nb batches of P
 ctd::FoldLast last_of(Phantom &P, int nb, bool keep_sums);
 // mean, standard error, avg RSD and deposited energy of nb folded batches
@@ -365,6 +363,8 @@ struct LaunchShape {
     int grid, block, threads_per_sm;
 };
 LaunchShape launch_shape(const ctd_ctx *ctx, const ctd::SharedTables &sh, int mode, bool trace);
+// one single-request launch of q on stream s
+int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, const LaunchShape &shape, cudaStream_t s);
 // q covers histories [h0, h1) of the problem of n histories in nb batches, deposits of
 // its first batch into tally and of each later one `stride` voxels further on, for a
 // launch of `warps` warps (`alone`: no other launch fills the SMs that it leaves idle)

@@ -83,6 +83,25 @@ def test_batched_chains_share_launches_like_plain_runs(ctd, contexts, lanes):
     ctd.ctd_destroy(c)
 
 
+@pytest.mark.parametrize("hist", [(9_001,) * 8, (900_000, 40_000, 30_011, 20_000, 9_000, 8_000, 5_003, 1_000),
+                                  (2, 3, 2_000_000, 100, 5_000, 33, 2, 7)])
+@pytest.mark.parametrize("threads", [0, 128])
+def test_chains_on_a_third_of_the_gpu_equal_plain_runs(ctd, contexts, hist, threads):
+    # eight chains: those with twice their histories still to be issued take a third of
+    # the blocks (alike, falling and dominated by one), at the default and another shape
+    ps = [I.head(n, 2, seed=50 + i, shape=(18 + i, 20, 14), d=1.0) for i, n in enumerate(hist)]
+    c = ctd.ctd_create(device=0, threads_per_block=threads, blocks_per_sm=7 if threads else 0)
+    hs = [ctd.load_problem(c, p) for p in ps]
+    ctd.ctd_run_batch(c, hs, [p.n_hist for p in ps], [p.seed for p in ps], 2)
+    for h, p in zip(hs, ps):
+        dose, sd, st = ctd.ctd_get_dose_and_stddev(c, h, p.phantom.nvox)
+        d1, s1, t1, h1 = ctd.run_problem(contexts[0], p)
+        ctd.ctd_destroy_phantom(contexts[0], h1)
+        assert [st[k] for k in COUNTS] == [t1[k] for k in COUNTS]
+        assert np.allclose(dose, d1, rtol=1e-12, atol=0)
+    ctd.ctd_destroy(c)
+
+
 @pytest.mark.parametrize("n_mat,e_max", [(1, 150), (16, 150), (16, 400), (16, 780)])
 def test_default_launch_shape_with_small_and_large_tables(ctd, contexts, n_mat, e_max):
     # blocks of 384 threads while three of them fit beside the attenuation tables, else
