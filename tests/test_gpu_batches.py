@@ -163,3 +163,24 @@ def test_groups_of_batches_of_a_large_grid(ctd, contexts):
     assert np.allclose(s0 ** 2, s1 ** 2, rtol=1e-9, atol=1e-12 * float((d0 ** 2).max()))
     assert t0["avg_rsd"] == pytest.approx(t1["avg_rsd"], rel=1e-9)
     assert t0["e_deposited_kev"] == pytest.approx(t1["e_deposited_kev"], rel=1e-12)
+
+
+@pytest.mark.parametrize("n_req", [1, 2, 3, 6])
+def test_served_requests_sharing_the_gpu_equal_plain_runs(ctd, contexts, n_req):
+    # three requests or more take a third of the blocks each; the last ones to run, and
+    # fewer, all of them and, alone, smaller claims
+    p = [I.head(1, seed=70 + i, shape=(18, 20, 14 + i), d=1.1) for i in range(n_req)]
+    B, k = 20_011, 4
+    c = ctd.ctd_create(device=0)
+    hs = [ctd.load_problem(c, x) for x in p]
+    ids = [ctd.ctd_submit(c, h, B, 0.0, x.seed, n_histories_max=(k + i) * B, min_batches=2)
+           for i, (h, x) in enumerate(zip(hs, p))]
+    for i in ids:
+        assert ctd.ctd_wait(c, i, 60.0)["state"] == ctd.REQ_DONE
+    for i, (h, x) in enumerate(zip(hs, p)):
+        dose, sd, st = ctd.ctd_get_dose_and_stddev(c, h, x.phantom.nvox)
+        d1, s1, t1, h1 = ctd.run_problem(contexts[0], I.scaled(x, n_hist=(k + i) * B, n_batches=k + i))
+        ctd.ctd_destroy_phantom(contexts[0], h1)
+        assert [st[q] for q in COUNTS] == [t1[q] for q in COUNTS]
+        assert np.allclose(dose, d1, rtol=1e-12, atol=0)
+    ctd.ctd_destroy(c)
