@@ -258,8 +258,11 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     }
     const void *work = ctx->u_work.p;
     put(&work, sizeof(work));
+    // (the descriptors hold what the transport and the folds take; the rest is what the last
+    // fold and the precision measures take, the densities among them: released buffers are
+    // handed out again one by one, so a phantom created anew may differ in these alone)
     for (int r = 0; r < n_req; ++r) {
-        const void *out[4] = {ps[r]->dose.p, ps[r]->sd.p, ps[r]->partials.p, ps[r]->result()};
+        const void *out[5] = {ps[r]->dose.p, ps[r]->sd.p, ps[r]->rho.p, ps[r]->partials.p, ps[r]->result()};
         put(out, sizeof(out));
     }
     // The batch loop is captured once into a CUDA graph and replayed while the
