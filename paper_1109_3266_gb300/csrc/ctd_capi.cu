@@ -4,17 +4,12 @@
 // the launch-shape search and the memory probes in ctd_tune.cu.
 #include <cuda_runtime.h>
 
-#include <sys/mman.h>
-#include <unistd.h>
-
 #include <algorithm>
-#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <thread>
 
 #include "ctd_host.h"
 
@@ -524,88 +519,6 @@ int prepare_run(ctd_ctx *ctx, Phantom &P, uint64_t n, int nb)
     if ((rc = build_tables(ctx, P))) return rc;
     if ((rc = upload_allocation(ctx, P, n, nb))) return rc;
     if ((rc = ensure_run_buffers(P))) return rc;
-    return CTD_OK;
-}
-
-// Device arrays read back into host memory the caller has just allocated: its pages
-// do not exist yet, and the copy itself (185 GB/s into existing pages) would wait for
-// the kernel to make them one by one, 4 ms for 134 MB.  A few threads make them, a
-// chunk at a time by writing one byte to each page of the destination (which the copy
-// overwrites), while the copies follow chunk by chunk.  Destinations that are small,
-// resident already (a reused or pinned buffer, by mincore) or not pageable memory are
-// copied as before.
-namespace {
-
-constexpr size_t kColdBytes = size_t(4) << 20, kReadChunk = size_t(8) << 20;
-
-// whether most of the n bytes at p are pages without memory behind them
-bool cold(const char *p, size_t n, size_t page)
-{
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p) & ~(page - 1);
-    const size_t pages = (reinterpret_cast<uintptr_t>(p) + n - a + page - 1) / page;
-    std::vector<unsigned char> in(pages);
-    if (mincore(reinterpret_cast<void *>(a), pages * page, in.data()) != 0) return false;
-    size_t there = 0;
-    for (unsigned char c : in) there += c & 1u;
-    return 2 * there < pages;
-}
-
-}  // namespace
-
-int read_back(ctd_ctx *ctx, const ReadPart *parts, int n_parts)
-{
-    struct Chunk {
-        char *dst;
-        const char *src;
-        size_t n;
-    };
-    const size_t page = static_cast<size_t>(sysconf(_SC_PAGESIZE));
-    size_t bytes = 0;
-    for (int i = 0; i < n_parts; ++i) bytes += parts[i].bytes;
-    std::vector<Chunk> chunks;
-    std::vector<std::thread> makers;
-    std::unique_ptr<std::atomic<int>[]> made;
-    std::atomic<size_t> next{0};
-    if (bytes >= kColdBytes) try {
-            bool any = false;
-            for (int i = 0; i < n_parts; ++i)
-                any = any || (parts[i].bytes >= page && cold(static_cast<char *>(parts[i].dst), parts[i].bytes, page));
-            if (any) {
-                for (int i = 0; i < n_parts; ++i)
-                    for (size_t o = 0; o < parts[i].bytes; o += kReadChunk)
-                        chunks.push_back({static_cast<char *>(parts[i].dst) + o, static_cast<const char *>(parts[i].src) + o,
-                                          std::min(kReadChunk, parts[i].bytes - o)});
-                made.reset(new std::atomic<int>[chunks.size()]());
-                const size_t hw = std::max(2u, std::thread::hardware_concurrency());
-                const size_t n = std::min({size_t(6), hw / 2, chunks.size()});
-                makers.reserve(n);
-                for (size_t t = 0; t < n; ++t)
-                    makers.emplace_back([&] {
-                        for (size_t k; (k = next.fetch_add(1)) < chunks.size();) {
-                            volatile char *p = chunks[k].dst;
-                            for (size_t o = 0; o < chunks[k].n; o += page) p[o] = 0;
-                            p[chunks[k].n - 1] = 0;
-                            made[k].store(1, std::memory_order_release);
-                        }
-                    });
-            }
-        } catch (const std::exception &) {
-            // no memory or no threads: what threads there are finish, the copies do not wait
-        }
-    cudaError_t e = cudaSuccess;
-    if (makers.empty()) {
-        for (int i = 0; i < n_parts && e == cudaSuccess; ++i)
-            e = cudaMemcpyAsync(parts[i].dst, parts[i].src, parts[i].bytes, cudaMemcpyDeviceToHost, ctx->stream);
-    } else {
-        for (size_t k = 0; k < chunks.size(); ++k) {
-            while (!made[k].load(std::memory_order_acquire)) std::this_thread::yield();
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(chunks[k].dst, chunks[k].src, chunks[k].n, cudaMemcpyDeviceToHost, ctx->stream);
-        }
-        for (std::thread &t : makers) t.join();
-    }
-    if (e != cudaSuccess) return fail(CTD_ECUDA, "cudaMemcpyAsync failed: %s", cudaGetErrorString(e));
-    CK(cudaStreamSynchronize(ctx->stream));
     return CTD_OK;
 }
 
