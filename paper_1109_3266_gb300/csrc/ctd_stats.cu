@@ -32,13 +32,15 @@ __device__ __forceinline__ void fold_voxel(double t, size_t v, double *__restric
 
 // Mean over nb batches and its standard error: s^2 = (sum d^2 - nb D^2) / (nb (nb - 1)),
 // nb D^2 as D sum d, with inv_nb = 1/nb and inv_nn = 1/(nb (nb - 1)).  (A comparison of
-// doubles is FP64 work too: the variance's sign and size are read from its bits.)
+// doubles is FP64 work too: the variance's sign and size are read from its bits.  What is
+// not a normal number above 2^-1000, such as an infinity or a NaN of tallies that are not
+// finite, takes the comparison.)
 __device__ __forceinline__ void mean_sd(double s1, double s2, double inv_nb, double inv_nn, double &D, double &sd)
 {
     D = s1 * inv_nb;
     const double var = fma(-D, s1, s2) * inv_nn;
-    const int hi = __double2hiint(var);
-    sd = hi >= ((1023 - 1000) << 20) ? root(var) : hi >= 0 ? sqrt(var) : 0.0;
+    const int hi = __double2hiint(var), lo = (1023 - 1000) << 20;
+    sd = static_cast<unsigned>(hi - lo) < static_cast<unsigned>(0x7ff00000 - lo) ? root(var) : var > 0.0 ? sqrt(var) : 0.0;
 }
 
 // Fold of a request's batches in one pass, and with kLast the mean, the standard
