@@ -124,14 +124,16 @@ __device__ __forceinline__ void block_sum(double (&x)[K])
 // a division per voxel.  Four quotients share one reciprocal: s0/D0 + s1/D1 =
 // (s0 D1 + s1 D0) / (D0 D1), and again for two such pairs, 3.5 FP64 operations a
 // voxel instead of 6 with a reciprocal each.  The doses are first scaled by a power
-// of two (on their exponent bits, exactly) that takes D_max to [2^-4, 2^-3), so no
-// product leaves the range; D_max outside [2^-1000, 2^1000] divides voxel by voxel.
+// of two (on their exponent bits, exactly) that takes D_max to [2^-4, 2^-3), so products
+// of doses stay in range; those with an error, down to 2^-22 of it, do while the error is
+// above 2^-1000.  D_max outside [2^-500, 2^500] divides voxel by voxel: inside, a smaller
+// error is below 2^-490 of its dose.
 __device__ __forceinline__ void rsd_sums(const double *__restrict__ dose, const double *__restrict__ sd,
                                          const float *__restrict__ rho, size_t nvox, double dmax, double *sums,
                                          int stride_out)
 {
     const long long lo1 = __double_as_longlong(0.1 * dmax), lo2 = __double_as_longlong(0.2 * dmax);
-    const bool scaled = dmax >= 0x1p-1000 && dmax <= 0x1p1000;
+    const bool scaled = dmax >= 0x1p-500 && dmax <= 0x1p500;
     const int shift = (__double2hiint(dmax) & 0x7ff00000) - ((1023 - 4) << 20);
     double rel = 0.0, s2 = 0.0;
     unsigned n1 = 0, n2 = 0;
