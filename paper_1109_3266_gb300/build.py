@@ -19,11 +19,13 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libctd.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 SOURCES = ["ctd_capi.cu", "ctd_forms.cu", "ctd_tune.cu", "ctd_transport.cu", "ctd_stats.cu", "ctd_physics.cpp",
-           "ctd_noalloc.cu", "ctd_probe.cu", "ctd_fluence.cu", "ctd_readback.cu"]
+           "ctd_noalloc.cu", "ctd_probe.cu", "ctd_fluence.cu", "ctd_readback.cpp"]
 HEADERS = ["ctd_internal.h", "ctd_host.h", "ctd_device.cuh", "ctd_stats.cuh"]
 FAST_MATH = {"ctd_transport.cu"}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-HOST_FLAGS = "-fPIC,-ffp-contract=off,-fno-fast-math,-O2"
+# (the host's table loops run 4 % slower or faster with where the linker puts them: a new
+# phantom's first call took 18.3 or 19.1 ms; aligned, 18.2)
+HOST_FLAGS = "-fPIC,-ffp-contract=off,-fno-fast-math,-O2,-falign-functions=64,-falign-loops=32"
 
 
 def nvcc() -> str:

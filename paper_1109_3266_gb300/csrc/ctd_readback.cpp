@@ -1,4 +1,4 @@
-// ctd_readback.cu -- results from device arrays into the caller's host memory.
+// ctd_readback.cpp -- results from device arrays into the caller's host memory.
 #include <cuda_runtime.h>
 
 #include <sys/mman.h>
