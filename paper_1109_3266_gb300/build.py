@@ -23,9 +23,9 @@ SOURCES = ["ctd_capi.cu", "ctd_forms.cu", "ctd_tune.cu", "ctd_transport.cu", "ct
 HEADERS = ["ctd_internal.h", "ctd_host.h", "ctd_device.cuh", "ctd_stats.cuh"]
 FAST_MATH = {"ctd_transport.cu"}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-# (the host's table loops run 4 % slower or faster with where the linker puts them: a new
-# phantom's first call took 18.3 or 19.1 ms; aligned, 18.2)
-HOST_FLAGS = "-fPIC,-ffp-contract=off,-fno-fast-math,-O2,-falign-functions=64,-falign-loops=32"
+# (the host's table loops run up to 5 % slower or faster with where the linker puts them: a
+# new phantom's first call took 18.3 or 19.1 ms; with loops on cache lines, 18.3)
+HOST_FLAGS = "-fPIC,-ffp-contract=off,-fno-fast-math,-O2,-falign-functions=64,-falign-loops=64"
 
 
 def nvcc() -> str:
