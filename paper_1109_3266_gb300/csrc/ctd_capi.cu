@@ -638,6 +638,7 @@ int ctd_create(ctd_ctx **out, const ctd_options *opt)
     CK(cudaGetDeviceCount(&ndev));
     if (ctx->device < 0 || ctx->device >= ndev) return fail(CTD_EINVAL, "device %d out of range (%d devices)", ctx->device, ndev);
     CK(cudaSetDevice(ctx->device));
+    ctx->buffers.attach(ctx->device);
     CK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
     if (ctx->l2_persist) {
         // the largest persisting set-aside the device grants, for this context's lifetime

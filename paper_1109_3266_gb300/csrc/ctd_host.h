@@ -11,6 +11,7 @@
 #include <cstdint>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -39,82 +40,44 @@ int fail(int code, const char *fmt, ...);
     } while (0)
 
 // Device buffers a context has released and may hand out again: the byte size of
-// each, up to `cap` bytes in all, and one block of scratch memory that a call borrows
+// each, up to kCap bytes in all, and one block of scratch memory that a call borrows
 // while it runs.  A phantom's buffers return here when it is destroyed (after its
 // context's stream is idle), so a phantom of the same size created next takes them
 // without cudaMalloc, and no cudaFree synchronises the device meanwhile.  The context
-// frees what is left when it is destroyed; what is idle is given back to the device
-// when an allocation finds no memory.
-struct BufferCache {
-    std::multimap<size_t, void *> blocks;
-    size_t cached = 0;
-    size_t cap = size_t(4) << 30;
-    void *scratch = nullptr;
-    size_t scratch_bytes = 0;
-    bool scratch_lent = false;
-    void *take(size_t bytes)
-    {
-        auto it = blocks.find(bytes);
-        if (it == blocks.end()) return nullptr;
-        void *p = it->second;
-        blocks.erase(it);
-        cached -= bytes;
-        return p;
-    }
-    bool give(void *p, size_t bytes)
-    {
-        if (cached + bytes > cap) return false;
-        blocks.emplace(bytes, p);
-        cached += bytes;
-        return true;
-    }
+// frees what is left when it is destroyed; what is idle here is given back to the device
+// when an allocation of this or another context of the process finds no memory
+// (device_allocate), which may run in another thread.
+class BufferCache {
+public:
+    static constexpr size_t kCap = size_t(4) << 30;
+    BufferCache() = default;
+    ~BufferCache();
+    void attach(int device);   // once, before the context has any buffer
+    int device() const { return device_; }
+    void *take(size_t bytes);
+    bool give(void *p, size_t bytes);
     // bytes that drop() would free
-    size_t idle() const { return cached + (scratch_lent ? 0 : scratch_bytes); }
-    void drop()
-    {
-        for (auto &b : blocks) cudaFree(b.second);
-        blocks.clear();
-        cached = 0;
-        drop_scratch();
-    }
-    void drop_scratch()
-    {
-        if (scratch_lent || !scratch) return;
-        cudaFree(scratch);
-        scratch = nullptr;
-        scratch_bytes = 0;
-    }
-    // cudaMalloc, once more after giving idle memory back
-    void *allocate(size_t bytes)
-    {
-        void *p = nullptr;
-        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
-        cudaGetLastError();
-        if (!idle()) return nullptr;
-        drop();
-        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
-        cudaGetLastError();
-        return nullptr;
-    }
+    size_t idle() const;
+    // frees what is idle; the bytes freed
+    size_t drop();
     // The scratch block, of at least `bytes` (it only grows); nullptr if it is lent
     // already or there is no memory.
-    void *borrow(size_t bytes)
-    {
-        if (scratch_lent) return nullptr;
-        if (scratch_bytes < bytes) {
-            drop_scratch();
-            if (!(scratch = allocate(bytes))) return nullptr;
-            scratch_bytes = bytes;
-        }
-        scratch_lent = true;
-        return scratch;
-    }
-    ~BufferCache()
-    {
-        scratch_lent = false;
-        drop();
-    }
+    void *borrow(size_t bytes);
+    void return_scratch();
+
+private:
+    mutable std::mutex lock_;
+    std::multimap<size_t, void *> blocks_;
+    size_t cached_ = 0;
+    void *scratch_ = nullptr;
+    size_t scratch_bytes_ = 0;
+    bool lent_ = false;
+    int device_ = -1;
 };
+
+// cudaMalloc on the current device, once more after its contexts' idle memory is given
+// back; nullptr if there is none
+void *device_allocate(size_t bytes);
 
 template <class T>
 struct DevBuf {
@@ -133,13 +96,8 @@ struct DevBuf {
         if (count <= n && p) return CTD_OK;
         release();
         if (count == 0) count = 1;
-        if (cache) {
-            p = static_cast<T *>(cache->take(count * sizeof(T)));
-            if (!p) p = static_cast<T *>(cache->allocate(count * sizeof(T)));
-        } else if (cudaMalloc(reinterpret_cast<void **>(&p), count * sizeof(T)) != cudaSuccess) {
-            cudaGetLastError();
-            p = nullptr;
-        }
+        if (cache) p = static_cast<T *>(cache->take(count * sizeof(T)));
+        if (!p) p = static_cast<T *>(device_allocate(count * sizeof(T)));
         if (!p) return fail(CTD_ENOMEM, "cudaMalloc of %zu bytes failed", count * sizeof(T));
         n = count;
         return CTD_OK;
@@ -222,7 +180,7 @@ struct Scratch {
     {
         if (!p) return;
         if (!idle) cudaStreamSynchronize(stream);
-        cache.scratch_lent = false;
+        cache.return_scratch();
     }
     bool borrow(size_t doubles) { return (p = static_cast<double *>(cache.borrow(doubles * sizeof(double)))) != nullptr; }
 };

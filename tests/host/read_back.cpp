@@ -59,6 +59,7 @@ cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 const char *cudaGetErrorString(cudaError_t) { return "fake"; }
 cudaError_t cudaFree(void *) { return cudaSuccess; }
+cudaError_t cudaGetDevice(int *) { return cudaSuccess; }
 cudaError_t cudaMalloc(void **, size_t) { return cudaErrorMemoryAllocation; }
 }
 

@@ -9,7 +9,7 @@ import host_unit
 
 @pytest.fixture(scope="module")
 def prog(tmp_path_factory):
-    return host_unit.program(tmp_path_factory, "read_back", "ctd_readback.cpp")
+    return host_unit.program(tmp_path_factory, "read_back", "ctd_readback.cpp", "ctd_memory.cpp")
 
 
 @pytest.mark.parametrize("n", [1 << 20, 2 << 20, (9 << 20) + 24, (33 << 20) + 8])
