@@ -169,7 +169,12 @@ const char *ctd_last_error(void);
 int ctd_abi_version(void);
 
 /* Context on one GPU.  opt may be NULL.  The context owns the stream it makes;
- * a stream passed in opt->stream stays the caller's. */
+ * a stream passed in opt->stream stays the caller's.
+ * Between calls a context keeps up to 4 GiB of device memory for reuse: the buffers
+ * of destroyed phantoms, and the scratch memory of its runs (at most 1 GiB) and
+ * batched calls (at most 4 GiB) as far as that leaves room.  It goes back to the
+ * device when an allocation of any context of the process on that device finds no
+ * memory, and with ctd_destroy; other users of the device cannot ask for it. */
 int ctd_create(ctd_ctx **out, const ctd_options *opt);
 int ctd_destroy(ctd_ctx *ctx);
 

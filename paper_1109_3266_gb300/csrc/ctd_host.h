@@ -40,8 +40,8 @@ int fail(int code, const char *fmt, ...);
     } while (0)
 
 // Device buffers a context has released and may hand out again: the byte size of
-// each, up to kCap bytes in all, and one block of scratch memory that a call borrows
-// while it runs.  A phantom's buffers return here when it is destroyed (after its
+// each, and one block of scratch memory that a call borrows while it runs; up to kCap
+// bytes in all while no call runs, the released buffers before the scratch.  A phantom's buffers return here when it is destroyed (after its
 // context's stream is idle), so a phantom of the same size created next takes them
 // without cudaMalloc, and no cudaFree synchronises the device meanwhile.  The context
 // frees what is left when it is destroyed; what is idle here is given back to the device
@@ -60,12 +60,13 @@ public:
     size_t idle() const;
     // frees what is idle; the bytes freed
     size_t drop();
-    // The scratch block, of at least `bytes` (it only grows); nullptr if it is lent
+    // The scratch block, of at least `bytes` (it grows only); nullptr if it is lent
     // already or there is no memory.
     void *borrow(size_t bytes);
     void return_scratch();
 
 private:
+    void *excess_scratch();
     mutable std::mutex lock_;
     std::multimap<size_t, void *> blocks_;
     size_t cached_ = 0;
@@ -207,8 +208,9 @@ struct ServeReq {
     bool in_flight = false, checked = false, split = false;
 };
 
-// device memory a plain run may take, while it runs, for the tallies of batches that
-// share a launch, and a batched call for all its requests'
+// device memory that a plain run may borrow for the tallies of batches that share a
+// launch, and a batched call for all its requests' (the context keeps it for the next
+// call, BufferCache)
 constexpr size_t kTallyBudget = size_t(1) << 30, kBatchTallyBudget = size_t(4) << 30;
 constexpr int kMaxLanes = 64;     // streams for request chains
 constexpr uint64_t kMaxTrace = 1ull << 26;   // histories of one trace call (16 B of device memory each)

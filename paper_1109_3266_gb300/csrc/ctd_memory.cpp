@@ -57,11 +57,26 @@ void *BufferCache::take(size_t bytes)
 
 bool BufferCache::give(void *p, size_t bytes)
 {
-    std::lock_guard<std::mutex> l(lock_);
-    if (cached_ + bytes > kCap) return false;
-    blocks_.emplace(bytes, p);
-    cached_ += bytes;
+    void *old = nullptr;
+    {
+        std::lock_guard<std::mutex> l(lock_);
+        if (cached_ + bytes > kCap) return false;
+        blocks_.emplace(bytes, p);
+        cached_ += bytes;
+        if (!lent_) old = excess_scratch();
+    }
+    if (old) cudaFree(old);
     return true;
+}
+
+// the scratch block, no longer the cache's, if it has no place beside the buffers
+void *BufferCache::excess_scratch()
+{
+    if (cached_ + scratch_bytes_ <= kCap) return nullptr;
+    void *p = scratch_;
+    scratch_ = nullptr;
+    scratch_bytes_ = 0;
+    return p;
 }
 
 size_t BufferCache::idle() const
@@ -114,8 +129,13 @@ void *BufferCache::borrow(size_t bytes)
 
 void BufferCache::return_scratch()
 {
-    std::lock_guard<std::mutex> l(lock_);
-    lent_ = false;
+    void *old;
+    {
+        std::lock_guard<std::mutex> l(lock_);
+        lent_ = false;
+        old = excess_scratch();
+    }
+    if (old) cudaFree(old);
 }
 
 void *device_allocate(size_t bytes)

@@ -124,6 +124,36 @@ static int kept()
     return 0;
 }
 
+// buffers and scratch together stay within what a context may keep, the buffers first
+static int bounded()
+{
+    const size_t G = size_t(1) << 30;
+    g_size = 64 * G;
+    EXPECT(BufferCache::kCap == 4 * G);
+    BufferCache a;
+    a.attach(0);
+    auto lend = [&](size_t bytes) {
+        Scratch s(a, nullptr);
+        return s.borrow(bytes / 8);
+    };
+    EXPECT(lend(4 * G) && a.idle() == 4 * G);      // alone: kept
+    release_into(a, G);                            // a released buffer takes its place
+    EXPECT(a.idle() == G && g_used[0] == G);
+    EXPECT(lend(3 * G) && a.idle() == 4 * G);      // just fits beside it
+    EXPECT(lend(3 * G + 8) && a.idle() == G);      // does not: given back when the call ends
+    {
+        Scratch s(a, nullptr);
+        EXPECT(s.borrow(2 * G / 8));
+        release_into(a, 2 * G);                    // released while it is lent
+        EXPECT(a.idle() == 3 * G && g_used[0] == 5 * G);
+    }
+    EXPECT(a.idle() == 3 * G && g_used[0] == 3 * G);
+    release_into(a, 2 * G);                        // the cached one, taken and released again
+    release_into(a, G + G / 2);                    // more than may be kept
+    EXPECT(a.idle() == 3 * G && g_used[0] == 3 * G);
+    return 0;
+}
+
 static int threads()
 {
     bool ok[2] = {false, false};
@@ -150,7 +180,7 @@ static int threads()
 int main(int, char **argv)
 {
     const std::string what = argv[1];
-    const int rc = what == "kept" ? kept() : what == "threads" ? threads() : given_back(what[0]);
+    const int rc = what == "kept" ? kept() : what == "bounded" ? bounded() : what == "threads" ? threads() : given_back(what[0]);
     if (rc) return rc;
     EXPECT(g_bad_frees == 0 && g_used[0] == 0 && g_used[1] == 0);
     std::puts("ok");
