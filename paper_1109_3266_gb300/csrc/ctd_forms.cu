@@ -49,11 +49,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     // longest processing time first), the k-th on stream k mod n_lanes.  Batches of a
     // request share launches as in a plain run, each with a tally in the call's scratch
     // memory; chains that share a stream share its part of that, which a fold leaves
-    // cleared for the next.  Fewer streams are used where the largest grids' tallies would
-    // not fit kBatchTallyBudget otherwise (two at least): 64 requests of 64^3 to 256^3
-    // voxels, 1.28e10 histories, took 1196 ms on 64 streams with most batches in launches
-    // of their own, 1056 ms on three with all of a request's in one, 1083 ms one ctd_run
-    // after another; 16 requests of 64^3 to 128^3 voxels 12.8, 7.7 and 9.7 ms.
+    // cleared for the next (plan_chains: the streams and the batches that share a launch).
     std::vector<int> order(n_req), step(n_req, 1);
     for (int r = 0; r < n_req; ++r) order[r] = r;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n_histories[a] > n_histories[b]; });
@@ -62,32 +58,20 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
     int n_lanes = std::min(n_req, ctx->batch_lanes);
     Scratch scratch(ctx->buffers, ctx->stream);
     if (!ctx->shared_launch) {
-        // voxels of scratch each of `lanes` streams needs for every batch of its requests,
-        // within an equal share of the budget
-        auto parts = [&](int lanes) {
-            std::vector<size_t> need(lanes, 0);
-            for (int k = 0; k < n_req; ++k) {
-                const int r = order[k];
-                step[r] = tallies_within(ps[r]->nvox, n_batches, kBatchTallyBudget / lanes);
-                if (step[r] > 1) need[k % lanes] = std::max(need[k % lanes], ps[r]->nvox * step[r]);
-            }
-            return need;
-        };
-        auto whole = [&] { return std::all_of(step.begin(), step.end(), [&](int g) { return g == n_batches; }); };
-        std::vector<size_t> need = parts(n_lanes);
-        while (!whole() && n_lanes > 2) need = parts(--n_lanes);
+        std::vector<size_t> nvox(n_req);
+        for (int k = 0; k < n_req; ++k) nvox[k] = ps[order[k]]->nvox;
+        const ChainPlan plan = plan_chains(nvox, n_batches, n_lanes, kBatchTallyBudget);
         size_t total = 0;
-        for (size_t v : need) total += v;
-        if (total && !scratch.borrow(total)) {
-            step.assign(n_req, 1);
-            n_lanes = std::min(n_req, ctx->batch_lanes);
-        }
-        if (scratch.p) {
+        for (size_t v : plan.need) total += v;
+        if (total && scratch.borrow(total)) {
+            n_lanes = plan.lanes;
             CK(cudaMemsetAsync(scratch.p, 0, total * sizeof(double), ctx->stream));
             std::vector<size_t> first(n_lanes, 0);
-            for (int l = 1; l < n_lanes; ++l) first[l] = first[l - 1] + need[l - 1];
-            for (int k = 0; k < n_req; ++k)
-                if (step[order[k]] > 1) tallies[order[k]] = scratch.p + first[k % n_lanes];
+            for (int l = 1; l < n_lanes; ++l) first[l] = first[l - 1] + plan.need[l - 1];
+            for (int k = 0; k < n_req; ++k) {
+                step[order[k]] = plan.group[k];
+                if (plan.group[k] > 1) tallies[order[k]] = scratch.p + first[k % n_lanes];
+            }
         }
     }
     // A chain's transport takes a third of the blocks per SM while the chains issued after

@@ -347,6 +347,38 @@ inline int tallies_within(size_t nvox, int nb, size_t budget)
     const size_t most = std::min(budget / (nvox * sizeof(double)), (static_cast<size_t>(1) << 32) / nvox);
     return static_cast<int>(std::min<size_t>(std::max<size_t>(most, 1), static_cast<size_t>(nb)));
 }
+// The request chains of a batched call, chain k of nvox[k] voxels (in the order of issue)
+// on stream k mod lanes: how many of a request's batches share a launch, and the voxels
+// of scratch that each stream's chains share for their tallies, `budget` bytes in all.
+struct ChainPlan {
+    int lanes;
+    std::vector<int> group;
+    std::vector<size_t> need;
+};
+// All of a request's batches share a launch, or as many as fit half the budget where they
+// need more (a grid that large would not get them all on any number of streams).  As many
+// streams as asked for are kept while the tallies of them all fit the budget, else fewer,
+// two at least: 64 requests of 64^3 to 256^3 voxels, 1.28e10 histories, took 1196 ms on 64
+// streams with most batches in launches of their own, 1056 ms on three with all of a
+// request's in one, 1083 ms one ctd_run after another.  The sum is what has to fit: with an
+// equal share for each stream one request of 256^3 voxels took 63 of 24^3 from 64 streams
+// to 3, 5.5 instead of 4.1 ms on the GPU, and 24 of 64^3 in 20 batches from 25 to 2, 10.2
+// instead of 8.0.
+inline ChainPlan plan_chains(const std::vector<size_t> &nvox, int n_batches, int lanes, size_t budget)
+{
+    const int n = static_cast<int>(nvox.size());
+    ChainPlan p{lanes, std::vector<int>(nvox.size()), {}};
+    const size_t part = budget / static_cast<size_t>(std::min(lanes, 2));
+    for (int k = 0; k < n; ++k) p.group[k] = tallies_within(nvox[k], n_batches, part);
+    for (;; --p.lanes) {
+        p.need.assign(p.lanes, 0);
+        for (int k = 0; k < n; ++k)
+            if (p.group[k] > 1) p.need[k % p.lanes] = std::max(p.need[k % p.lanes], nvox[k] * p.group[k]);
+        size_t total = 0;
+        for (size_t v : p.need) total += v;
+        if (total <= budget / sizeof(double) || p.lanes <= 2) return p;
+    }
+}
 // fold of batches [b0, b0 + k) of the problem of n histories in nb batches from tally[k][nvox]
 ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, double *tally, bool clear);
 // one transport launch over histories [h0, h1) of n in nb batches (set_range), bracketed
