@@ -463,13 +463,10 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
     const int nb = R.batches + std::max(n, 1);
     ctd::SharedTables sh{};
     fill_shared(P, sh);
-    // Batches that do not fill the GPU, of three requests or more, take a third of the
-    // blocks per SM each, so that three launches share every SM and one's tail, fold and stop
-    // test lie under the others' transport: eight requests of 4e6 histories a batch 107.1 ->
-    // 102.9 ms; arriving at 60 /s, p99 0.45 -> 0.33 s at the same p50.  (With the first in
-    // line on the whole GPU 104.0 ms; two requests at a third each would leave SMs idle.)
+    std::vector<double> running;
+    for (int64_t id : ctx->active) running.push_back(static_cast<double>(ctx->sreqs[id].req.batch_histories));
     LaunchShape shape = launch_shape(ctx, sh, q.mode, false);
-    if (ctx->active.size() >= 3 && static_cast<double>(B) < fill_histories(ctx))
+    if (shares_sms(static_cast<double>(B), running, fill_histories(ctx)))
         shape.grid = ctx->num_sms * std::max(shape.grid / ctx->num_sms / 3, 1);
     const int warps = shape.grid * (shape.block / 32);
     // from min_batches on the last of these batches is followed by the stop test

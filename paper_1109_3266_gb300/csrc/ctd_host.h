@@ -379,6 +379,20 @@ inline ChainPlan plan_chains(const std::vector<size_t> &nvox, int n_batches, int
         if (total <= budget / sizeof(double) || p.lanes <= 2) return p;
     }
 }
+// Whether a batch of a served request takes a third of the blocks per SM, so that three
+// launches share every SM and one's tail, fold and stop test lie under the others'
+// transport: batches that do not fill the GPU (`fill` histories), while three requests of
+// such batches or more run (`running`: the batches of all that do, this one's among them).
+// Eight requests of 4e6 histories a batch 107.1 -> 102.9 ms; arriving at 60 /s, p99 0.45 ->
+// 0.33 s at the same p50.  (With the first in line on the whole GPU 104.0 ms; two requests
+// at a third each would leave SMs idle.)  Beside requests that fill the GPU a small one
+// keeps the whole grid, as the first in line should: a request of 24 batches of 4e6
+// beside two and three such took 49.4 and 49.2 ms (on a third 50.7 and 52.4), one of 1e6 a
+// batch 36.7 and 36.3 (38.4 and 37.4).
+inline bool shares_sms(double batch, const std::vector<double> &running, double fill)
+{
+    return batch < fill && std::count_if(running.begin(), running.end(), [&](double b) { return b < fill; }) >= 3;
+}
 // fold of batches [b0, b0 + k) of the problem of n histories in nb batches from tally[k][nvox]
 ctd::FoldBatches fold_of(const Phantom &P, uint64_t n, int nb, int b0, int k, double *tally, bool clear);
 // one transport launch over histories [h0, h1) of n in nb batches (set_range), bracketed
