@@ -174,7 +174,7 @@ int ctd_run_batch(ctd_ctx *ctx, int n_req, const ctd_phantom *phantoms, const ui
                     const size_t d = static_cast<size_t>(b) * n_req + r;
                     const int g = std::min(step[r], n_batches - b);
                     // (a fold clears the tallies for what follows on the stream)
-                    e = launch_one(ctx, P, descs[d], shapes[r], ls);
+                    e = launch_one(ctx, P, descs[d], shapes[r], n_lanes == 1, ls);
                     if (e == CTD_OK)
                         e = ctd::launch_fold(fold_of(P, n_histories[r], n_batches, b, g, tallies[r], true), P.rinv.p,
                                              P.sum_d.p, P.sum_d2.p, P.edep.p, P.nvox, b == 0,
@@ -469,6 +469,7 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
     if (shares_sms(static_cast<double>(B), running, fill_histories(ctx)))
         shape.grid = ctx->num_sms * std::max(shape.grid / ctx->num_sms / 3, 1);
     const int warps = shape.grid * (shape.block / 32);
+    const bool alone = ctx->active.size() == 1;
     // from min_batches on the last of these batches is followed by the stop test
     const int done = R.batches + n;
     R.checked = n > 0 && done >= R.req.min_batches;
@@ -478,10 +479,9 @@ int launch_work(ctd_ctx *ctx, ServeReq &R, Phantom &P, bool first_in_line)
         const uint64_t first = static_cast<uint64_t>(R.batches + j) * B;
         const uint64_t h0 = j == 0 ? first + lo : first, h1 = j == 0 ? first + hi : first + B;
         if (h0 < h1) {
-            set_range(q, B * nb, nb, h0, h1, P.tally.p, 0, ctx->chunk, warps,
-                      ctx->active.size() == 1);
+            set_range(q, B * nb, nb, h0, h1, P.tally.p, 0, ctx->chunk, warps, alone);
             CK(cudaMemsetAsync(q.work, 0, sizeof(unsigned long long), s));
-            CKS(launch_one(ctx, P, q, shape, s));
+            CKS(launch_one(ctx, P, q, shape, alone, s));
             hist += static_cast<double>(h1 - h0);
         }
         if (j < n)

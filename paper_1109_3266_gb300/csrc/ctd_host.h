@@ -324,15 +324,16 @@ struct LaunchShape {
 };
 LaunchShape launch_shape(const ctd_ctx *ctx, const ctd::SharedTables &sh, int mode, bool trace);
 // one single-request launch of q on stream s
-int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, const LaunchShape &shape, cudaStream_t s);
+int launch_one(ctd_ctx *ctx, Phantom &P, const ctd::RequestDesc &q, const LaunchShape &shape, bool alone,
+               cudaStream_t s);
 // q covers histories [h0, h1) of the problem of n histories in nb batches, deposits of
 // its first batch into tally and of each later one `stride` voxels further on, for a
 // launch of `warps` warps (`alone`: no other launch fills the SMs that it leaves idle)
 void set_range(ctd::RequestDesc &q, uint64_t n, int nb, uint64_t h0, uint64_t h1, double *tally, uint32_t stride,
                int chunk, int warps, bool alone);
 // launches L (one request, its range set) on s, in pieces whose histories share the
-// upper word of their index; the claim counter is at 0
-int launch_single(const ctd_ctx *ctx, ctd::LaunchParams &L, const LaunchShape &shape, cudaStream_t s,
+// upper word of their index (`alone` as in set_range); the claim counter is at 0
+int launch_single(const ctd_ctx *ctx, ctd::LaunchParams &L, const LaunchShape &shape, bool alone, cudaStream_t s,
                   const ctd::L2Window *win = nullptr);
 // batch b of n histories in nb batches: its first history
 inline uint64_t batch_start(uint64_t n, int nb, int b)
