@@ -381,7 +381,7 @@ int finish_stats(Phantom &P, int nb, cudaStream_t s)
 
 // The launch shape of a single request.  The default residency of 4 blocks of 256
 // threads per SM becomes 3 of 384 in full transport: 36 warps instead of 32 at 56
-// registers (54 used, no spills; blocks of a multiple of 128 threads load the four
+// registers (all used, no spills; blocks of a multiple of 128 threads load the four
 // schedulers alike).  Per 2e8 histories CBCT water 15.00 -> 14.93 ms, head 24.70 ->
 // 24.25, per 1e8 a 4 mm head 17.77 -> 17.45 (40 warps spill: 24.84).  Runs that limit
 // the real interactions are source-bound and stay (4.70 against 4.84 ms), as do shapes

@@ -1,7 +1,8 @@
 // ctd_host.h -- host-side state behind the C ABI of include/ctd.h, shared by
 // ctd_capi.cu (contexts, phantoms, set-up, the plain form, results),
-// ctd_forms.cu (the batched and served forms) and ctd_tune.cu (launch-shape
-// search, memory probes).
+// ctd_forms.cu (the batched and served forms), ctd_tune.cu (launch-shape
+// search, memory probes), ctd_claims.cpp (the histories of a launch),
+// ctd_memory.cpp (device memory) and ctd_readback.cpp (results into host memory).
 #pragma once
 
 #include <cuda_runtime.h>
